@@ -31,6 +31,7 @@
 
 #include "df.cuh"
 #include "fast.h"
+#include "fx.cuh"
 #include "kernels.cuh"
 
 namespace fsp {
@@ -137,6 +138,8 @@ template <typename T, int D, bool PK = false> struct RD {
             return C{-a.x, -a.y};
         } else if constexpr (m == 24) {
             return D < 0 ? cmuli(a) : cmulmi(a);
+        } else if constexpr (std::is_same<T, fx>::value) {
+            return fx_w32<D, m>(a);
         } else {
             constexpr T c = T(cos32(m)), s = T(D * sin32(m));
             return cmul(a, C{c, s});
@@ -842,16 +845,6 @@ FSP_CFG(float, 256, 16, 16, 16, 16, 1)
 FSP_CFG(float, 512, 32, 16, 16, 32, 1)
 FSP_CFG(float, 1024, 16, 16, 16, 16, 4)
 FSP_CFG(float, 2048, 16, 8, 16, 16, 8)  // column passes of non-cubic boxes only (an axis of 1024)
-FSP_CFG(double, 32, 8, 16, 4, 8, 1)
-FSP_CFG(double, 48, 12, 8, 4, 3, 4)
-FSP_CFG(double, 96, 24, 8, 4, 3, 8)
-FSP_CFG(double, 192, 24, 8, 8, 3, 8)
-FSP_CFG(double, 384, 24, 8, 8, 6, 8)
-FSP_CFG(double, 64, 8, 16, 8, 8, 1)
-FSP_CFG(double, 128, 16, 8, 8, 16, 1)
-FSP_CFG(double, 256, 16, 8, 16, 16, 1)
-FSP_CFG(double, 512, 8, 8, 8, 8, 8)
-FSP_CFG(double, 1024, 16, 8, 16, 8, 8)
 FSP_CFG(df, 32, 8, 16, 4, 8, 1)
 FSP_CFG(df, 64, 8, 16, 8, 8, 1)
 FSP_CFG(df, 128, 16, 8, 8, 16, 1)

@@ -19,6 +19,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
 #include <utility>
 
 namespace fsp {
@@ -161,14 +162,24 @@ template <typename T, int D> struct Dft {
     }
 };
 
+// entries of a roots table: complex values of the working type, except for
+// the fixed-point engine (fx.cuh)
+template <typename T> struct tw_of { using t = cx_t<T>; };
+template <typename T> using fx_tw_t = typename tw_of<T>::t;
+
 template <typename T, int D> struct Engine {
     using C = cx_t<T>;
+    using TW = fx_tw_t<T>;
 
-    // exp(D 2 pi i e / n) from the forward table tw[e] = exp(-2 pi i e / n)
-    static __device__ __forceinline__ C twid(const C *__restrict__ tw, int e) {
-        C w = tw[e];
-        if (D > 0) w.y = -w.y;
-        return w;
+    // x exp(D 2 pi i e / n) from the forward table tw[e] = exp(-2 pi i e / n)
+    static __device__ __forceinline__ C twiddle(C x, const TW *__restrict__ tw, int e) {
+        if constexpr (std::is_same<TW, C>::value) {
+            C w = tw[e];
+            if (D > 0) w.y = -w.y;
+            return cmul(x, w);
+        } else {
+            return tw_of<T>::template mul<D>(x, tw[e]);  // divided by 4
+        }
     }
 
     // The loops over butterflies and over the radix are unrolled by
@@ -176,7 +187,7 @@ template <typename T, int D> struct Engine {
     // persistent batched kernel) pragma unrolling is not guaranteed, and a
     // partially unrolled loop would send the register array v to local memory.
     template <int R>
-    static __device__ __forceinline__ void stage(C *buf, int ld, int n, int Ns, const C *__restrict__ tw, int l,
+    static __device__ __forceinline__ void stage(C *buf, int ld, int n, int Ns, const TW *__restrict__ tw, int l,
                                                  int sub, int tpl, bool act) {
         constexpr int KMAX = kMaxV / R;
         const int nb = n / R;
@@ -202,10 +213,12 @@ template <typename T, int D> struct Engine {
             const int b = sub + k * tpl;
             if (act && b < nb) {
                 const int j = b % Ns;
-                if (j != 0) {
+                // fixed point: every stage but the first divides by 4
+                if (std::is_same<TW, C>::value ? j != 0 : Ns > 1) {
+                    if constexpr (!std::is_same<TW, C>::value) v[k * R] = tw_of<T>::quarter(v[k * R]);
                     Unroll<1, R>::run([&](auto rc) {
                         constexpr int r = decltype(rc)::value;
-                        v[k * R + r] = cmul(v[k * R + r], twid(tw, r * j * tws));
+                        v[k * R + r] = twiddle(v[k * R + r], tw, r * j * tws);
                     });
                 }
                 if constexpr (R == 2) Dft<T, D>::r2(v + k * R);
@@ -225,7 +238,7 @@ template <typename T, int D> struct Engine {
 
     // Transform all lines held in buf in place.  Every thread of the CTA must
     // call this (it contains barriers); `act` only gates the arithmetic.
-    static __device__ __forceinline__ void run(C *buf, int ld, const Stages &st, const C *__restrict__ tw, int l,
+    static __device__ __forceinline__ void run(C *buf, int ld, const Stages &st, const TW *__restrict__ tw, int l,
                                                int sub, int tpl, bool act) {
         int Ns = 1;
         for (int s = 0; s < st.n5; ++s, Ns *= 5) stage<5>(buf, ld, st.n, Ns, tw, l, sub, tpl, act);

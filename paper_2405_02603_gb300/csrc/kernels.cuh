@@ -72,8 +72,8 @@ template <typename T, int IN, int OUT, int MODE> cudaError_t launch_lines(const 
 template <typename T> cudaError_t launch_r2c_rows(const RowsArgs &a, cudaStream_t s);
 template <typename T> cudaError_t launch_c2r_rows(const RowsArgs &a, cudaStream_t s);
 
-// exp(-2 pi i e / n), e in [0,n), computed in double precision (sincospi) and
-// rounded to T.
+// exp(-2 pi i e / n), e in [0,n): computed in double precision (sincospi) and
+// rounded to T; for double the fixed-point roots of fx.cuh, 62 fraction bits.
 template <typename T> cudaError_t launch_roots(void *tw, int n, cudaStream_t s);
 
 }  // namespace fsp

@@ -1,11 +1,116 @@
 // kernels_impl.cuh -- definitions of the line-transform kernels (included once
 // per real type by kernels_f32.cu / kernels_f64.cu).
+//
+// FP64 lines (T = double) are transformed in 64-bit fixed point (fx.cuh): the
+// doubles of a tile are loaded into shared memory as they are, tile_scale
+// turns them into integers at their line's scale, and the store turns the
+// results back.  Where a kernel has the two forms, W is the working type and
+// FX says which form it is.
 #pragma once
+#include "fast.cuh"
+#include "fx_line.cuh"
 #include "kernels.cuh"
 
 namespace fsp {
 
 constexpr int kMaxThreads = 512;
+constexpr int kMaxLines = 32;  // lines per CTA (lgL <= 5)
+
+template <typename T> struct work_of {
+    using t = T;
+};
+template <> struct work_of<double> {
+    using t = fx;
+};
+template <int D> struct Dft<fx, D> {
+    using C = cfx;
+    static __device__ __forceinline__ void r2(C *v) { fast::RD<fx, D>::template dft<2, false, false>(v); }
+    static __device__ __forceinline__ void r3(C *v) { fast::RD<fx, D>::template dft<3, false, false>(v); }
+    static __device__ __forceinline__ void r4(C *v) { fast::RD<fx, D>::template dft<4, false, false>(v); }
+    static __device__ __forceinline__ void r5(C *v) { fast::RD<fx, D>::template dft<5, false, false>(v); }
+    static __device__ __forceinline__ void r8(C *v) { fast::RD<fx, D>::template dft<8, false, false>(v); }
+};
+
+// Per line of a tile: the largest upper word and the 1-norm in units of
+// 2^(em - 16) (integers, so that the order of the atomics does not matter),
+// the largest modulus of a product with S, and the scale of the results.
+struct TileLines {
+    int hmax[kMaxLines], mmax[kMaxLines];
+    unsigned sum[kMaxLines], sum2[kMaxLines];
+    int hS[kMaxLines];
+    int eo[kMaxLines];
+    bool bad[kMaxLines];
+};
+__device__ __forceinline__ void tile_clear(TileLines &q) {
+    if (threadIdx.x < kMaxLines) {
+        q.hmax[threadIdx.x] = q.mmax[threadIdx.x] = q.hS[threadIdx.x] = 0;
+        q.sum[threadIdx.x] = q.sum2[threadIdx.x] = 0;
+    }
+}
+// s <= 2^em * (some 2^12) in units of 2^(em - 16), rounded up; |em| < 100
+__device__ __forceinline__ unsigned tile_units(float s, int em) {
+    return (unsigned)(s * __int_as_float((127 + 16 - em) << 23)) + 1u;
+}
+// fx_ke of a runtime schedule (5s, 3s, 8s, last): modulus <= 2^B after every
+// stage, each stage after the first dividing by 4 beforehand
+__device__ __forceinline__ int tile_ke(const Stages &st, int em, int eL, int B) {
+    int eb = -100000, g = 0, d = 0;
+    auto stage = [&](int grow) {
+        g += grow;
+        eb = max(eb, min(em + 1 + g, eL) - d);
+        d += 2;
+    };
+    for (int i = 0; i < st.n5; ++i) stage(3);
+    for (int i = 0; i < st.n3; ++i) stage(2);
+    for (int i = 0; i < st.n8; ++i) stage(3);
+    if (st.last) stage(st.last == 4 ? 2 : 1);
+    return B - max(eb, min(em + 1, eL));  // (a transform of length 1 has no stage)
+}
+__device__ __forceinline__ int tile_log2(const Stages &st) {
+    return 3 * st.n5 + 2 * st.n3 + 3 * st.n8 + (st.last == 4 ? 2 : st.last == 2 ? 1 : 0) + 1;
+}
+// twice the number of stages that divide by 4
+__device__ __forceinline__ int tile_div(const Stages &st) {
+    return 2 * max(st.n5 + st.n3 + st.n8 + (st.last ? 1 : 0) - 1, 0);
+}
+// Turns the doubles at positions p < np of line l into integers; every thread
+// of the CTA calls it after the barrier that ends the loads, and a barrier
+// follows.  The result's scale is that of the integers.
+__device__ __forceinline__ FxScale tile_scale(cfx *buf, int ld, int np, const Stages &st, int B, int l, int sub,
+                                              int tpl, bool act, TileLines &q) {
+    float s = 0.f;
+    int h = 0;
+    if (act) {
+        for (int p = sub; p < np; p += tpl) fx_bound(buf[p * ld + l], s, h);
+        atomicMax(&q.hmax[l], h);
+    }
+    __syncthreads();
+    h = q.hmax[l];
+    const int em = fx_em(h);
+    FxScale sc;
+    sc.any = fx_far(em), sc.bad = (h >> 20) == 0x7ff;
+    if (act && !sc.any) atomicAdd(&q.sum[l], tile_units(s, em));
+    __syncthreads();
+    const int eL = sc.any ? em + tile_log2(st) : em - 16 + fx_clog2(1.5f * (float)q.sum[l] + 1e-30f);
+    sc.ke = tile_ke(st, em, eL, B);
+    if (act)
+        for (int p = sub; p < np; p += tpl) buf[p * ld + l] = fx_conv<true, false>(buf[p * ld + l], sc);
+    return sc;
+}
+// a double or a float as the real part of a working value, still unscaled
+__device__ __forceinline__ fx tile_real(double x) { return fx(__double_as_longlong(x), 0); }
+__device__ __forceinline__ float tile_real(float x) { return x; }
+__device__ __forceinline__ cfx tile_cplx(double2 q) { return fx_raw(q); }
+__device__ __forceinline__ float2 tile_cplx(float2 q) { return q; }
+// a result of line l for the store
+__device__ __forceinline__ double2 tile_out(const cfx &v, const TileLines &q, int l) {
+    return FxOut<true, false>(q.eo[l], q.bad[l])(v);
+}
+__device__ __forceinline__ double tile_out_re(const cfx &v, const TileLines &q, int l) {
+    return FxOut<true, true>(q.eo[l], q.bad[l]).template one<true>(v.x.v);
+}
+__device__ __forceinline__ float2 tile_out(float2 v, const TileLines &, int) { return v; }
+__device__ __forceinline__ float tile_out_re(float2 v, const TileLines &, int) { return v.x; }
 
 // Loads of data another CTA of the same launch may have written (the
 // persistent batched kernel) bypass L1, which is not coherent across SMs.
@@ -21,7 +126,12 @@ template <bool COH, typename V> __device__ __forceinline__ V ldw(const V *p) {
 // Every thread of the CTA must call it (barriers); threads beyond L*tpl idle.
 template <typename T, int IN, int OUT, int MODE, bool COH>
 __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long by, unsigned char *smem_raw) {
-    using C = cx_t<T>;
+    using W = typename work_of<T>::t;
+    using C = cx_t<W>;
+    using IC = cx_t<T>;
+    constexpr bool FX = std::is_same<W, fx>::value;
+    __shared__ TileLines tl;
+    if constexpr (FX) tile_clear(tl);
     C *buf = reinterpret_cast<C *>(smem_raw);
     const int L = 1 << a.lgL, lmask = L - 1;
     const int ld = L + 1;
@@ -34,7 +144,7 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
     // issued before their shared-memory stores, so that several are in flight
     constexpr int U = 4;
     if (IN == IN_CPLX) {
-        const C *in = reinterpret_cast<const C *>(a.in) + b * a.in_batch;
+        const IC *in = reinterpret_cast<const IC *>(a.in) + b * a.in_batch;
         const int cnt = L * a.n_in;
         if (a.in_line == 1) {
             for (int base = tid; base < cnt; base += U * nth) {
@@ -42,9 +152,9 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int idx = base + u * nth, l = idx & lmask, p = idx >> a.lgL;
-                    q[u] = C{T(0), T(0)};
+                    q[u] = C{W(0), W(0)};
                     if (idx < cnt && line0 + l < a.nlines)
-                        q[u] = ldw<COH>(in + ((long long)(line0 + l) + (long long)p * a.in_pos));
+                        q[u] = tile_cplx(ldw<COH>(in + ((long long)(line0 + l) + (long long)p * a.in_pos)));
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
@@ -58,9 +168,9 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int idx = base + u * nth, p = idx % a.n_in, l = idx / a.n_in;
-                    q[u] = C{T(0), T(0)};
+                    q[u] = C{W(0), W(0)};
                     if (idx < cnt && line0 + l < a.nlines)
-                        q[u] = ldw<COH>(in + ((long long)(line0 + l) * a.in_line + (long long)p * a.in_pos));
+                        q[u] = tile_cplx(ldw<COH>(in + ((long long)(line0 + l) * a.in_line + (long long)p * a.in_pos)));
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
@@ -70,7 +180,7 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
             }
         }
         const int zc = L * (n - a.n_in);
-        for (int idx = tid; idx < zc; idx += nth) buf[(a.n_in + (idx >> a.lgL)) * ld + (idx & lmask)] = C{T(0), T(0)};
+        for (int idx = tid; idx < zc; idx += nth) buf[(a.n_in + (idx >> a.lgL)) * ld + (idx & lmask)] = C{W(0), W(0)};
     } else {
         // DCT-I through the DFT of the even extension: y[j] = x[j] for j <= M,
         // y[2M - j] = x[j] for 0 < j < M.  DST-I through the DFT of
@@ -92,11 +202,11 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
             if (line0 + l < a.nlines) x = ldw<COH>(in + ((long long)(line0 + l) * a.in_line + (long long)p * a.in_pos));
             const bool inner = p > 0 && p < M;
             if (IN == IN_REAL_EVEN) {
-                buf[p * ld + l] = C{x, T(0)};
-                if (inner) buf[(n - p) * ld + l] = C{x, T(0)};
+                buf[p * ld + l] = C{tile_real(x), W(0)};
+                if (inner) buf[(n - p) * ld + l] = C{tile_real(x), W(0)};
             } else {
-                buf[p * ld + l] = C{T(0), inner ? x : T(0)};
-                if (inner) buf[(n - p) * ld + l] = C{T(0), -x};
+                buf[p * ld + l] = C{W(0), tile_real(inner ? x : T(0))};
+                if (inner) buf[(n - p) * ld + l] = C{W(0), tile_real(-x)};
             }
         }
     }
@@ -104,11 +214,18 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
 
     const int l = tid & lmask, sub = tid >> a.lgL;
     const bool act = (line0 + l) < a.nlines && sub < a.tpl;
-    const C *tw = reinterpret_cast<const C *>(a.tw);
+    const fx_tw_t<W> *tw = reinterpret_cast<const fx_tw_t<W> *>(a.tw);
+    FxScale sc{};
+    if constexpr (FX) {
+        sc = tile_scale(buf, ld, IN == IN_CPLX ? a.n_in : n, a.st, MODE == M_FWD_MUL_INV ? 61 : 62, l, sub, a.tpl, act,
+                        tl);
+        if (MODE != M_FWD_MUL_INV && act && sub == 0) tl.eo[l] = tile_div(a.st) - sc.ke, tl.bad[l] = sc.bad;
+        __syncthreads();
+    }
     if (MODE == M_INV)
-        Engine<T, +1>::run(buf, ld, a.st, tw, l, sub, a.tpl, act);
+        Engine<W, +1>::run(buf, ld, a.st, tw, l, sub, a.tpl, act);
     else
-        Engine<T, -1>::run(buf, ld, a.st, tw, l, sub, a.tpl, act);
+        Engine<W, -1>::run(buf, ld, a.st, tw, l, sub, a.tpl, act);
 
     if (MODE == M_FWD_MUL_INV) {
         const T *S = reinterpret_cast<const T *>(a.S);
@@ -117,6 +234,38 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
         const int fy = (int)b <= hb ? (int)b : 2 * hb - (int)b;
         const int cnt = L * n;
         const int odd = a.odd;
+        if constexpr (FX) {
+            // as k_fx_col: bounds of the products, then the products at the
+            // scale of the inverse
+            const double *Sl = S + (long long)fy * a.s_batch + line0 + l;
+            float s2 = 0.f, m2 = 0.f;
+            int hS = 0;
+            if (act) {
+                for (int p = sub; p < n; p += a.tpl)
+                    fx_bound_mul(buf[p * ld + l], Sl[(long long)(p <= a.half ? p : h2 - p) * a.s_pos], s2, m2, hS);
+                atomicMax(&tl.hS[l], hS);
+                atomicMax(&tl.mmax[l], __float_as_int(m2));
+            }
+            __syncthreads();
+            const int eS = fx_es(tl.hS[l]);
+            const bool near = fx_near(eS), bad = sc.bad || eS == 1025;
+            // products' moduli are below 2^em (near: in units of 2^32)
+            const int ef = fx_clog2(1.1f * __int_as_float(tl.mmax[l]));
+            const int em = near ? ef + 32 : 61 + eS;
+            if (act && near) atomicAdd(&tl.sum2[l], tile_units(s2, ef));
+            __syncthreads();
+            const int eL = near ? em - 16 + fx_clog2(1.1f * (float)tl.sum2[l] + 1e-30f) : em + tile_log2(a.st);
+            const int ke = min(tile_ke(a.st, em - 1, eL, 62), 60 - em);
+            const int neg_b = odd == 2 && (int)b > hb ? -1 : 0, neg_z = odd == 1 ? -1 : 0;
+            if (act) {
+                for (int p = sub; p < n; p += a.tpl) {
+                    const cfx q = fx_mul_s(buf[p * ld + l], Sl[(long long)(p <= a.half ? p : h2 - p) * a.s_pos], ke,
+                                           neg_b ^ (p > a.half ? neg_z : 0), near);
+                    buf[p * ld + l] = odd == 0 ? q : cfx{q.y, -q.x};
+                }
+                if (sub == 0) tl.eo[l] = 2 * tile_div(a.st) - sc.ke - ke, tl.bad[l] = bad;
+            }
+        } else {
         const T sb = odd == 2 && (int)b > hb ? T(-1) : T(1);
         for (int idx = tid; idx < cnt; idx += nth) {
             const int ll = idx & lmask, p = idx >> a.lgL;
@@ -136,15 +285,16 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
                 buf[p * ld + ll] = v;
             }
         }
+        }
         __syncthreads();
-        Engine<T, +1>::run(buf, ld, a.st, tw, l, sub, a.tpl, act);
+        Engine<W, +1>::run(buf, ld, a.st, tw, l, sub, a.tpl, act);
     }
 
     // ---- store (crop to n_out positions)
     const int cnt = L * a.n_out;
     const bool col = (a.out_line == 1);
     if (OUT == OUT_CPLX) {
-        C *out = reinterpret_cast<C *>(a.out) + b * a.out_batch;
+        IC *out = reinterpret_cast<IC *>(a.out) + b * a.out_batch;
         for (int idx = tid; idx < cnt; idx += nth) {
             int ll, p;
             if (col) {
@@ -154,7 +304,8 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
                 p = idx % a.n_out;
                 ll = idx / a.n_out;
             }
-            if (line0 + ll < a.nlines) out[(long long)(line0 + ll) * a.out_line + (long long)p * a.out_pos] = buf[p * ld + ll];
+            if (line0 + ll < a.nlines)
+                out[(long long)(line0 + ll) * a.out_line + (long long)p * a.out_pos] = tile_out(buf[p * ld + ll], tl, ll);
         }
     } else {
         T *out = reinterpret_cast<T *>(a.out) + b * a.out_batch;
@@ -168,7 +319,7 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
                 ll = idx / a.n_out;
             }
             if (line0 + ll < a.nlines)
-                out[(long long)(line0 + ll) * a.out_line + (long long)p * a.out_pos] = buf[p * ld + ll].x;
+                out[(long long)(line0 + ll) * a.out_line + (long long)p * a.out_pos] = tile_out_re(buf[p * ld + ll], tl, ll);
         }
     }
 }
@@ -187,7 +338,12 @@ __global__ void __launch_bounds__(kMaxThreads) k_lines(const LinesArgs a) {
 //   X[k] = E + w^k O,  X[N-k] = conj(E - w^k O),  w = exp(-2 pi i / 2N).
 template <typename T, bool COH>
 __device__ __forceinline__ void r2c_tile(const RowsArgs &a, int bx, unsigned char *smem_raw) {
-    using C = cx_t<T>;
+    using W = typename work_of<T>::t;
+    using C = cx_t<W>;
+    using IC = cx_t<T>;
+    constexpr bool FX = std::is_same<W, fx>::value;
+    __shared__ TileLines tl;
+    if constexpr (FX) tile_clear(tl);
     C *buf = reinterpret_cast<C *>(smem_raw);
     const int L = 1 << a.lgL, lmask = L - 1, ld = L + 1;
     const int tid = threadIdx.x, nth = blockDim.x;
@@ -202,14 +358,14 @@ __device__ __forceinline__ void r2c_tile(const RowsArgs &a, int bx, unsigned cha
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int idx = base + u * nth, m = idx % Mh, l = idx / Mh;
-            q[u] = C{T(0), T(0)};
+            q[u] = C{W(0), W(0)};
             if (idx < cnt && row0 + l < a.nrows) {
                 const T *xr = x + (row0 + l) * a.x_row;
                 if ((N & 1) == 0) {
-                    q[u] = ldw<COH>(reinterpret_cast<const C *>(xr) + m);
+                    q[u] = tile_cplx(ldw<COH>(reinterpret_cast<const IC *>(xr) + m));
                 } else {
-                    q[u].x = ldw<COH>(xr + 2 * m);
-                    q[u].y = (2 * m + 1 < N) ? ldw<COH>(xr + 2 * m + 1) : T(0);
+                    q[u].x = tile_real(ldw<COH>(xr + 2 * m));
+                    q[u].y = tile_real((2 * m + 1 < N) ? ldw<COH>(xr + 2 * m + 1) : T(0));
                 }
             }
         }
@@ -220,24 +376,36 @@ __device__ __forceinline__ void r2c_tile(const RowsArgs &a, int bx, unsigned cha
         }
     }
     const int zc = L * (N - Mh);
-    for (int idx = tid; idx < zc; idx += nth) buf[(Mh + (idx >> a.lgL)) * ld + (idx & lmask)] = C{T(0), T(0)};
+    for (int idx = tid; idx < zc; idx += nth) buf[(Mh + (idx >> a.lgL)) * ld + (idx & lmask)] = C{W(0), W(0)};
     __syncthreads();
 
     const int l = tid & lmask, sub = tid >> a.lgL;
     const bool act = (row0 + l) < a.nrows && sub < a.tpl;
-    Engine<T, -1>::run(buf, ld, a.st, reinterpret_cast<const C *>(a.tw), l, sub, a.tpl, act);
+    if constexpr (FX) {
+        const FxScale sc = tile_scale(buf, ld, Mh, a.st, 61, l, sub, a.tpl, act, tl);
+        // the coefficients below come out at half their scale
+        if (act && sub == 0) tl.eo[l] = tile_div(a.st) - sc.ke + 1, tl.bad[l] = sc.bad;
+        __syncthreads();
+    }
+    Engine<W, -1>::run(buf, ld, a.st, reinterpret_cast<const fx_tw_t<W> *>(a.tw), l, sub, a.tpl, act);
 
-    const C *tw2 = reinterpret_cast<const C *>(a.tw2);
+    const fx_tw_t<W> *tw2 = reinterpret_cast<const fx_tw_t<W> *>(a.tw2);
     if (act) {
         for (int k = sub; 2 * k <= N; k += a.tpl) {
             const int kc = (k == 0) ? 0 : N - k;
             const C zk = buf[k * ld + l], zc = buf[kc * ld + l];
-            const C e = C{T(0.5) * (zk.x + zc.x), T(0.5) * (zk.y - zc.y)};
-            const C o = C{T(0.5) * (zk.y + zc.y), T(-0.5) * (zk.x - zc.x)};
-            const C wo = cmul(tw2[k], o);
+            C e, wo;
+            if constexpr (FX) {  // a quarter of the sums: X / 2
+                e = C{fx_quarter(zk.x + zc.x), fx_quarter(zk.y - zc.y)};
+                wo = fx_twiddle<-1>(C{zk.y + zc.y, zc.x - zk.x}, tw2[k]);
+            } else {
+                e = C{T(0.5) * (zk.x + zc.x), T(0.5) * (zk.y - zc.y)};
+                const C o = C{T(0.5) * (zk.y + zc.y), T(-0.5) * (zk.x - zc.x)};
+                wo = k == 0 ? o : cmul(tw2[k], o);
+            }
             if (k == 0) {
-                buf[0 * ld + l] = cadd(e, o);
-                buf[N * ld + l] = csub(e, o);
+                buf[0 * ld + l] = cadd(e, wo);
+                buf[N * ld + l] = csub(e, wo);
             } else {
                 buf[k * ld + l] = cadd(e, wo);
                 if (2 * k != N) buf[kc * ld + l] = cconj(csub(e, wo));
@@ -246,11 +414,11 @@ __device__ __forceinline__ void r2c_tile(const RowsArgs &a, int bx, unsigned cha
     }
     __syncthreads();
 
-    C *c = reinterpret_cast<C *>(a.c);
+    IC *c = reinterpret_cast<IC *>(a.c);
     const int np = N + 1, cnt2 = L * np;
     for (int idx = tid; idx < cnt2; idx += nth) {
         const int k = idx % np, ll = idx / np;
-        if (row0 + ll < a.nrows) c[(row0 + ll) * a.c_row + k] = buf[k * ld + ll];
+        if (row0 + ll < a.nrows) c[(row0 + ll) * a.c_row + k] = tile_out(buf[k * ld + ll], tl, ll);
     }
 }
 
@@ -267,13 +435,18 @@ template <typename T> __global__ void __launch_bounds__(kMaxThreads) k_r2c_rows(
 //   z = IFFT_N(Z) (unnormalised),  y[2m] = Re z[m],  y[2m+1] = Im z[m].
 template <typename T, bool COH>
 __device__ __forceinline__ void c2r_tile(const RowsArgs &a, int bx, unsigned char *smem_raw) {
-    using C = cx_t<T>;
+    using W = typename work_of<T>::t;
+    using C = cx_t<W>;
+    using IC = cx_t<T>;
+    constexpr bool FX = std::is_same<W, fx>::value;
+    __shared__ TileLines tl;
+    if constexpr (FX) tile_clear(tl);
     C *buf = reinterpret_cast<C *>(smem_raw);
     const int L = 1 << a.lgL, ld = L + 1;
     const int tid = threadIdx.x, nth = blockDim.x;
     const long long row0 = (long long)bx << a.lgL;
     const int N = a.N, np = N + 1;
-    const C *c = reinterpret_cast<const C *>(a.c);
+    const IC *c = reinterpret_cast<const IC *>(a.c);
 
     const int cnt = L * np;
     constexpr int U = 4;  // loads in flight per thread
@@ -282,8 +455,8 @@ __device__ __forceinline__ void c2r_tile(const RowsArgs &a, int bx, unsigned cha
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int idx = base + u * nth, k = idx % np, l = idx / np;
-            q[u] = C{T(0), T(0)};
-            if (idx < cnt && row0 + l < a.nrows) q[u] = ldw<COH>(c + ((row0 + l) * a.c_row + k));
+            q[u] = C{W(0), W(0)};
+            if (idx < cnt && row0 + l < a.nrows) q[u] = tile_cplx(ldw<COH>(c + ((row0 + l) * a.c_row + k)));
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -295,20 +468,33 @@ __device__ __forceinline__ void c2r_tile(const RowsArgs &a, int bx, unsigned cha
 
     const int l = tid & (L - 1), sub = tid >> a.lgL;
     const bool act = (row0 + l) < a.nrows && sub < a.tpl;
-    const C *tw2 = reinterpret_cast<const C *>(a.tw2);
+    const fx_tw_t<W> *tw2 = reinterpret_cast<const fx_tw_t<W> *>(a.tw2);
+    if constexpr (FX) {
+        // the inputs' bounds hold for Z / 4 (|Z| / 4 <= the mean of |X[k]| and |X[N-k]|)
+        const FxScale sc = tile_scale(buf, ld, np, a.st, 62, l, sub, a.tpl, act, tl);
+        if (act && sub == 0) tl.eo[l] = tile_div(a.st) + 2 - sc.ke, tl.bad[l] = sc.bad;
+        __syncthreads();
+    }
     if (act) {
         for (int k = sub; 2 * k <= N; k += a.tpl) {
             const int kc = N - k;
             const C xk = buf[k * ld + l], xc = buf[kc * ld + l];
-            const C A = C{xk.x + xc.x, xk.y - xc.y};
-            const C B = C{xk.x - xc.x, xk.y + xc.y};
-            const C w = tw2[k];
-            buf[k * ld + l] = cadd(A, cmuli(cmul(cconj(w), B)));
-            if (k != 0 && 2 * k != N) buf[kc * ld + l] = cadd(cconj(A), cmuli(cmul(w, cconj(B))));
+            if constexpr (FX) {  // Z / 4; i w^k conj B = conj(-i conj(w^k) B)
+                const C A = C{fx_quarter(xk.x + xc.x), fx_quarter(xk.y - xc.y)};
+                const C wb = fx_twiddle<+1>(C{xk.x - xc.x, xk.y + xc.y}, tw2[k]);
+                buf[k * ld + l] = C{A.x - wb.y, A.y + wb.x};
+                if (k != 0 && 2 * k != N) buf[kc * ld + l] = C{A.x + wb.y, wb.x - A.y};
+            } else {
+                const C A = C{xk.x + xc.x, xk.y - xc.y};
+                const C B = C{xk.x - xc.x, xk.y + xc.y};
+                const C w = tw2[k];
+                buf[k * ld + l] = cadd(A, cmuli(cmul(cconj(w), B)));
+                if (k != 0 && 2 * k != N) buf[kc * ld + l] = cadd(cconj(A), cmuli(cmul(w, cconj(B))));
+            }
         }
     }
     __syncthreads();
-    Engine<T, +1>::run(buf, ld, a.st, reinterpret_cast<const C *>(a.tw), l, sub, a.tpl, act);
+    Engine<W, +1>::run(buf, ld, a.st, reinterpret_cast<const fx_tw_t<W> *>(a.tw), l, sub, a.tpl, act);
 
     T *x = reinterpret_cast<T *>(const_cast<void *>(a.x));
     const int Mh = (N + 1) >> 1, cnt2 = L * Mh;
@@ -316,9 +502,9 @@ __device__ __forceinline__ void c2r_tile(const RowsArgs &a, int bx, unsigned cha
         const int m = idx % Mh, ll = idx / Mh;
         if (row0 + ll < a.nrows) {
             T *xr = x + (row0 + ll) * a.x_row;
-            const C v = buf[m * ld + ll];
+            const IC v = tile_out(buf[m * ld + ll], tl, ll);
             if ((N & 1) == 0) {
-                reinterpret_cast<C *>(xr)[m] = v;
+                reinterpret_cast<IC *>(xr)[m] = v;
             } else {
                 xr[2 * m] = v.x;
                 if (2 * m + 1 < N) xr[2 * m + 1] = v.y;
@@ -388,14 +574,16 @@ template <typename T> cudaError_t launch_roots(void *tw, int n, cudaStream_t s) 
     return cudaGetLastError();
 }
 
-#define FSP_INSTANTIATE(T)                                                                          \
+#define FSP_INSTANTIATE_PASSES(T)                                                                   \
     template cudaError_t launch_lines<T, IN_CPLX, OUT_CPLX, M_FWD>(const LinesArgs &, cudaStream_t); \
     template cudaError_t launch_lines<T, IN_CPLX, OUT_CPLX, M_INV>(const LinesArgs &, cudaStream_t); \
     template cudaError_t launch_lines<T, IN_CPLX, OUT_CPLX, M_FWD_MUL_INV>(const LinesArgs &, cudaStream_t); \
     template cudaError_t launch_r2c_rows<T>(const RowsArgs &, cudaStream_t);                         \
     template cudaError_t launch_c2r_rows<T>(const RowsArgs &, cudaStream_t);                         \
-    template cudaError_t launch_roots<T>(void *, int, cudaStream_t);                                 \
     template size_t lines_smem_bytes<T>(const LinesArgs &);                                          \
     template size_t rows_smem_bytes<T>(const RowsArgs &);
+#define FSP_INSTANTIATE(T)                                                                          \
+    FSP_INSTANTIATE_PASSES(T)                                                                       \
+    template cudaError_t launch_roots<T>(void *, int, cudaStream_t);
 
 }  // namespace fsp
