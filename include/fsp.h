@@ -348,10 +348,11 @@ typedef struct fsp_batch fsp_batch;
  * phi[i] (16-byte aligned, N_i^3 reals).  The plans must be distinct (each
  * owns its workspace), live, of one dtype and on the current device; they
  * must outlive the batch.  The work list and the graph are built once; each
- * launch re-reads rho[i] and rewrites phi[i].  Every tile uses the generic
- * mixed-radix engine with the plan's tile shapes, so a batched result is
- * bitwise equal to a single solve through that engine (FSP_GENERIC_ONLY=1).
- * Synchronises `stream`. */
+ * launch re-reads rho[i] and rewrites phi[i].  FP32 plans that all have
+ * specialised kernels (N = 32 .. 256) run those; otherwise every tile uses the
+ * generic mixed-radix engine with the plan's tile shapes, and a batched result
+ * is bitwise equal to a single solve through that engine
+ * (FSP_GENERIC_ONLY=1).  Synchronises `stream`. */
 fsp_status fsp_batch_create(fsp_batch **out, fsp_plan *const *plans, const void *const *rho, void *const *phi,
                             int count, fsp_stream stream);
 /* Launch the batch's graph on `stream` (asynchronous).  One launch of a batch

@@ -24,6 +24,7 @@
 
 #include "../../include/fsp.h"
 #include "batch.h"
+#include "batch_fast.h"
 #include "fast_field.h"
 #include "df.cuh"
 #include "fast.h"
@@ -1609,6 +1610,12 @@ struct fsp_batch {
     BatchCtl *d_ctl = nullptr;
     size_t ctl_bytes = 0;
     BatchLaunch launch{};
+    // every plan on the specialised FP32 kernels: their own persistent kernel
+    bool fast = false;
+    bool tuning = false;  // the autotuner at work: it times the generic engine's shapes
+    FastBatchSolve *d_fsolves = nullptr;
+    FastBatchItem *d_items = nullptr;
+    FastBatchLaunch flaunch{};
     double timeout_ms = 1000.0;
     int form = 0;  // 0: one persistent kernel; 1: the solves' own launches on several streams
     cudaGraph_t graph = nullptr;
@@ -1625,11 +1632,16 @@ bool batch_live(const fsp_batch *b) {
     return b && g_batches.count(b) && b->magic == kBatchMagic;
 }
 
+void batch_free_lists(fsp_batch *b) {
+    for (void *q : {(void *)b->d_solves, (void *)b->d_segs, (void *)b->d_ctl, (void *)b->d_fsolves, (void *)b->d_items})
+        if (q) dev_free(q);
+    b->d_solves = nullptr, b->d_segs = nullptr, b->d_ctl = nullptr, b->d_fsolves = nullptr, b->d_items = nullptr;
+}
+
 void batch_free(fsp_batch *b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
-    for (void *q : {(void *)b->d_solves, (void *)b->d_segs, (void *)b->d_ctl})
-        if (q) dev_free(q);
+    batch_free_lists(b);
     b->magic = 0;
     delete b;
 }
@@ -1671,10 +1683,30 @@ BatchSolve batch_solve_of(const fsp_plan *p, const void *rho, void *phi, const T
     return b;
 }
 
+// The same for the specialised FP32 kernels: the arguments of
+// enqueue_solve_fast's launches.
+FastBatchSolve fast_batch_solve_of(const fsp_plan *p, const void *rho, void *phi) {
+    const int N = p->N;
+    const long long P = p->P;
+    FastBatchSolve b{};
+    b.N = N;
+    fast::RowArgs r{};
+    r.x = rho, r.c = p->W1, r.x_row = N, r.c_row = P, r.nrows = N * N, r.tw = p->tw_n, r.tw2 = p->tw_2n;
+    b.r1 = b.r5 = r;
+    b.r5.x = phi;
+    fast::ColArgs a{};
+    a.tw = p->tw_2n, a.nlines = N + 1;
+    b.c2 = b.c3 = b.c4 = a;
+    b.c2.in = p->W1, b.c2.out = p->W2;
+    b.c3.in = b.c3.out = p->W2, b.c3.S = p->S, b.c3.half = N;
+    b.c4.in = p->W2, b.c4.out = p->W1;
+    return b;
+}
+
 fsp_status batch_build_graph(fsp_batch *b) {
     if (b->exec) cudaGraphExecDestroy(b->exec), b->exec = nullptr;
     if (b->graph) cudaGraphDestroy(b->graph), b->graph = nullptr;
-    b->launch.timeout_ns = (unsigned long long)(b->timeout_ms * 1e6);
+    b->launch.timeout_ns = b->flaunch.timeout_ns = (unsigned long long)(b->timeout_ms * 1e6);
     cudaStream_t cs;
     if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return FSP_ECUDA;
     // form 1: kStreams capture streams forked from cs; a plan's solves stay on
@@ -1694,8 +1726,9 @@ fsp_status batch_build_graph(fsp_batch *b) {
         cudaError_t e1 = cudaMemsetAsync(b->d_ctl, 0, b->ctl_bytes, cs);
         cudaError_t e2 = e1;
         if (e1 == cudaSuccess && b->form == 0) {
-            e2 = b->dtype == FSP_F64 ? launch_batch_kernel<double>(b->launch, cs)
-                                     : launch_batch_kernel<float>(b->launch, cs);
+            e2 = b->fast               ? launch_fast_batch(b->flaunch, cs)
+                 : b->dtype == FSP_F64 ? launch_batch_kernel<double>(b->launch, cs)
+                                       : launch_batch_kernel<float>(b->launch, cs);
         } else if (e1 == cudaSuccess) {
             e2 = cudaEventRecord(fev[kStreams], cs);
             for (int i = 0; i < kStreams && e2 == cudaSuccess; ++i) e2 = cudaStreamWaitEvent(fs[i], fev[kStreams], 0);
@@ -1740,9 +1773,64 @@ void batch_tiles(const fsp_batch *b, const fsp_plan *p, TileCfg &row, TileCfg &c
     if (choose_tile(2 * p->N, c.tpl, csize, it->second.second, c.lgL)) col = c;
 }
 
+// batch_build for plans that are all on the specialised FP32 kernels.
+fsp_status batch_build_fast(fsp_batch *b, cudaStream_t s) {
+    const int count = b->count;
+    std::vector<FastBatchSolve> solves;
+    std::vector<FastBatchItem> items;
+    std::vector<int> order(count);
+    size_t smem = 0;
+    for (int i = 0; i < count; ++i) {
+        order[i] = i;
+        solves.push_back(fast_batch_solve_of(b->plans[i], b->rho[i], b->phi[i]));
+        smem = std::max(smem, fast_batch_smem(b->plans[i]->N));
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->plans[x]->N > b->plans[y]->N; });
+    b->segs.clear();
+    for (int pass = 0; pass < 5; ++pass)
+        for (int i : order) {
+            int ntiles[5], group[5];
+            fast_batch_tiles(b->plans[i]->N, ntiles, group);
+            auto count_of = [&](int p) { return (ntiles[p] + group[p] - 1) / group[p]; };
+            BatchSeg g{};
+            g.solve = i, g.pass = pass, g.first = (int)items.size(), g.ntiles = ntiles[pass];
+            g.need_prev = pass ? count_of(pass - 1) : 0;
+            for (int t = 0; t < ntiles[pass]; t += group[pass]) items.push_back({(int)b->segs.size(), t});
+            b->segs.push_back(g);
+        }
+    b->total = (int)items.size();
+    b->ctl_bytes = sizeof(BatchCtl) + sizeof(int) * (5 * (size_t)count);
+    DevBuf ds, dg, dc, di;
+    fsp_status st;
+    if ((st = alloc_or_nomem(ds, sizeof(FastBatchSolve) * count)) != FSP_OK) return st;
+    if ((st = alloc_or_nomem(dg, sizeof(BatchSeg) * b->segs.size())) != FSP_OK) return st;
+    if ((st = alloc_or_nomem(dc, b->ctl_bytes)) != FSP_OK) return st;
+    if ((st = alloc_or_nomem(di, sizeof(FastBatchItem) * items.size())) != FSP_OK) return st;
+    b->d_fsolves = (FastBatchSolve *)ds.release(), b->d_segs = (BatchSeg *)dg.release();
+    b->d_ctl = (BatchCtl *)dc.release(), b->d_items = (FastBatchItem *)di.release();
+    if (cudaMemcpyAsync(b->d_fsolves, solves.data(), sizeof(FastBatchSolve) * count, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyAsync(b->d_segs, b->segs.data(), sizeof(BatchSeg) * b->segs.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyAsync(b->d_items, items.data(), sizeof(FastBatchItem) * items.size(), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return FSP_ECUDA;
+    const int per_sm = fast_batch_blocks_per_sm(smem);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device);
+    if (per_sm < 1 || sms < 1) return FSP_EUNSUPPORTED;
+    FastBatchLaunch &L = b->flaunch;
+    L.solves = b->d_fsolves, L.segs = b->d_segs, L.items = b->d_items, L.total = b->total, L.ctl = b->d_ctl;
+    L.grid = (unsigned)std::min<long long>((long long)sms * per_sm, b->total), L.smem = smem;
+    return batch_build_graph(b);
+}
+
 // (Re)build descriptors, work list, device arrays and graph of a batch.
 fsp_status batch_build(fsp_batch *b, cudaStream_t s) {
     const int count = b->count;
+    batch_free_lists(b);
+    b->fast = b->dtype == FSP_F32_MIXED && !b->tuning &&
+              std::all_of(b->plans.begin(), b->plans.end(),
+                          [](const fsp_plan *p) { return p->fast && p->W1 && fast_batch_has(p->N); });
+    if (b->fast) return batch_build_fast(b, s);
     const size_t csize = 2 * b->plans[0]->rsize;
     b->solves.clear();
     b->segs.clear();
@@ -1772,9 +1860,6 @@ fsp_status batch_build(fsp_batch *b, cudaStream_t s) {
             b->segs.push_back(g);
         }
     b->total = first;
-    for (void *q : {(void *)b->d_solves, (void *)b->d_segs, (void *)b->d_ctl})
-        if (q) dev_free(q);
-    b->d_solves = nullptr, b->d_segs = nullptr, b->d_ctl = nullptr;
     b->ctl_bytes = sizeof(BatchCtl) + sizeof(int) * (5 * (size_t)count);
     DevBuf ds, dg, dc;
     fsp_status st;
@@ -1898,11 +1983,9 @@ double time_batch(fsp_batch *b, cudaStream_t s, int reps) {
     cudaMemcpy(&status, &b->d_ctl->status, sizeof(int), cudaMemcpyDeviceToHost);
     return (e == cudaSuccess && status == 0) ? best : -1.0;
 }
-}  // namespace
 
-extern "C" fsp_status fsp_batch_autotune(fsp_batch *b, fsp_stream stream) {
-    if (!batch_live(b)) return FSP_EINVAL;
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+// Coordinate descent over the generic engine's tile shapes of a batch.
+fsp_status batch_tune(fsp_batch *b, cudaStream_t s) {
     std::vector<int> Ns;
     for (auto *p : b->plans)
         if (std::find(Ns.begin(), Ns.end(), p->N) == Ns.end()) Ns.push_back(p->N);
@@ -1934,6 +2017,17 @@ extern "C" fsp_status fsp_batch_autotune(fsp_batch *b, fsp_stream stream) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     for (auto &kv : b->shape) g_tuning[{kv.first, (int)b->dtype}] = kv.second;
     return FSP_OK;
+}
+}  // namespace
+
+extern "C" fsp_status fsp_batch_autotune(fsp_batch *b, fsp_stream stream) {
+    if (!batch_live(b)) return FSP_EINVAL;
+    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    b->tuning = true;
+    const fsp_status tuned = batch_tune(b, s);
+    b->tuning = false;
+    const fsp_status built = b->dtype == FSP_F32_MIXED ? batch_build(b, s) : FSP_OK;
+    return tuned != FSP_OK ? tuned : built;
 }
 
 extern "C" fsp_status fsp_batch_destroy(fsp_batch *b) {

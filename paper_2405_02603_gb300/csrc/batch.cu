@@ -1,5 +1,7 @@
 // batch.cu -- many independent solves of mixed sizes in one persistent launch
-// (the batched systems form; the paper solves one grid at a time).
+// (the batched systems form; the paper solves one grid at a time), on the
+// generic engine: FP64 batches and FP32 ones with a size that has no
+// specialised kernels (the others: batch_fast_f32.cu).
 //
 // Work list: every solve contributes 5 segments (P1..P5) of tiles; segments
 // are ordered pass-major (all P1 segments, then all P2, ...).  Each CTA of the

@@ -479,20 +479,21 @@ template <typename T, int MODE, int n> struct ColOpt {
 // compiler's code differs between the forms; each pass takes the one it
 // measured fastest with.
 template <typename T, int n, int V, int L, int R1, int R2, int R3, int MODE, bool RG>
-__device__ __forceinline__ void fast_col_body(const ColArgs &a) {
+__device__ __forceinline__ void fast_col_body(const ColArgs &a, unsigned bx, unsigned by) {
 #include "fast_col_body.inc"
 }
 template <typename T, int n, int V, int L, int R1, int R2, int R3, int MODE, bool RG = false>
 __global__ void __launch_bounds__(L *(n / V)) k_fast_col(const ColArgs a) {
+    const unsigned bx = blockIdx.x, by = blockIdx.y;
 #include "fast_col_body.inc"
 }
 template <typename T, int n, int V, int L, int R1, int R2, int R3, int MODE, bool RG = false>
 __global__ void __launch_bounds__(L *(n / V), 2) k_fast_col_occ2(const ColArgs a) {
-    fast_col_body<T, n, V, L, R1, R2, R3, MODE, RG>(a);
+    fast_col_body<T, n, V, L, R1, R2, R3, MODE, RG>(a, blockIdx.x, blockIdx.y);
 }
 template <typename T, int n, int V, int L, int R1, int R2, int R3, int MODE, bool RG = false>
 __global__ void __launch_bounds__(L *(n / V)) k_fast_col_inl(const ColArgs a) {
-    fast_col_body<T, n, V, L, R1, R2, R3, MODE, RG>(a);
+    fast_col_body<T, n, V, L, R1, R2, R3, MODE, RG>(a, blockIdx.x, blockIdx.y);
 }
 template <typename T, int n, int V, int L, int R1, int R2, int R3, int MODE, bool RG>
 constexpr auto col_kernel() {
@@ -509,7 +510,7 @@ constexpr auto col_kernel() {
 // P1: rows of N reals -> N+1 coefficients of the zero-padded length-2N row,
 // through the length-N FFT of z[m] = x[2m] + i x[2m+1] (zero for m >= N/2).
 template <typename T, int N, int V, int L, int R1, int R2, int R3>
-__global__ void __launch_bounds__(L *(N / V)) k_fast_r2c(const RowArgs a) {
+__device__ __forceinline__ void fast_r2c_tile(const RowArgs &a, unsigned bx) {
     using C = cx_t<T>;
     constexpr int TPL = N / V, LD = L + 1, NTH = L * TPL, H = N / 2;
     static_assert(NTH % 32 == 0, "row kernels use whole warps per row");
@@ -517,7 +518,7 @@ __global__ void __launch_bounds__(L *(N / V)) k_fast_r2c(const RowArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *buf = reinterpret_cast<C *>(smem_raw);
     const int tid = threadIdx.x, l = tid % L, t = tid / L;
-    const long long row0 = (long long)blockIdx.x * L;
+    const long long row0 = (long long)bx * L;
     using R = typename io_of<T>::t;
     const R *x = reinterpret_cast<const R *>(a.x);
     // coalesced row loads of the packed pairs (x[2m], x[2m+1]), m < N/2, all
@@ -580,17 +581,21 @@ __global__ void __launch_bounds__(L *(N / V)) k_fast_r2c(const RowArgs a) {
         }
     }
 }
+template <typename T, int N, int V, int L, int R1, int R2, int R3>
+__global__ void __launch_bounds__(L *(N / V)) k_fast_r2c(const RowArgs a) {
+    fast_r2c_tile<T, N, V, L, R1, R2, R3>(a, blockIdx.x);
+}
 
 // P5: N+1 coefficients -> first N of the 2N real outputs.
-template <typename T, int N, int V, int L, int R1, int R2, int R3>
-__global__ void __launch_bounds__(L *(N / V)) k_fast_c2r(const RowArgs a) {
+template <typename T, int N, int V, int L, int R1, int R2, int R3, bool COH>
+__device__ __forceinline__ void fast_c2r_tile(const RowArgs &a, unsigned bx) {
     using C = cx_t<T>;
     constexpr int TPL = N / V, LD = L + 1, NTH = L * TPL, H = N / 2;
     constexpr int RL = LastR<R1, R2, R3>::value;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *buf = reinterpret_cast<C *>(smem_raw);
     const int tid = threadIdx.x, l = tid % L, t = tid / L;
-    const long long row0 = (long long)blockIdx.x * L;
+    const long long row0 = (long long)bx * L;
     // one warp per row: coalesced loads of the N+1 coefficients, all of a
     // thread's loads issued before the first shared-memory store
     const C *c = reinterpret_cast<const C *>(a.c);
@@ -606,7 +611,7 @@ __global__ void __launch_bounds__(L *(N / V)) k_fast_c2r(const RowArgs a) {
 #pragma unroll
             for (int j = 0; j < KPL; ++j) {
                 const int k = lane + 32 * j;
-                q[i * KPL + j] = okr && k <= N ? crow[k] : C{T(0), T(0)};
+                q[i * KPL + j] = okr && k <= N ? (COH ? ldcg_c(crow + k) : crow[k]) : C{T(0), T(0)};
             }
         }
 #pragma unroll
@@ -651,6 +656,10 @@ __global__ void __launch_bounds__(L *(N / V)) k_fast_c2r(const RowArgs a) {
         const int m = idx % H, rr = idx / H;
         if (row0 + rr < a.nrows) store_pair<T>(x + (row0 + rr) * N, m, buf[m * LD + rr]);
     }
+}
+template <typename T, int N, int V, int L, int R1, int R2, int R3>
+__global__ void __launch_bounds__(L *(N / V)) k_fast_c2r(const RowArgs a) {
+    fast_c2r_tile<T, N, V, L, R1, R2, R3, false>(a, blockIdx.x);
 }
 
 // ------------------------------------ row kernels, one lane per position --
@@ -711,13 +720,13 @@ __device__ __forceinline__ void lane_row_stages(cx_t<T> *v, cx_t<T> *buf, int t,
 
 // P1, lane per position: same arithmetic as k_fast_r2c
 template <typename T, int N, int V, int L, int R1>
-__global__ void __launch_bounds__(L *(N / V), (lane_row_minb<N, V, L>())) k_lane_r2c(const RowArgs a) {
+__device__ __forceinline__ void lane_r2c_tile(const RowArgs &a, unsigned bx) {
     using C = cx_t<T>;
     constexpr int TPL = N / V;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *buf = reinterpret_cast<C *>(smem_raw);
     const int tid = threadIdx.x, t = tid % TPL, l = tid / TPL;
-    const long long row = (long long)blockIdx.x * L + l;
+    const long long row = (long long)bx * L + l;
     const bool live = row < a.nrows;
     using R = typename io_of<T>::t;
     const R *xr = reinterpret_cast<const R *>(a.x) + (live ? row : 0) * N;
@@ -757,22 +766,26 @@ __global__ void __launch_bounds__(L *(N / V), (lane_row_minb<N, V, L>())) k_lane
         }
     }
 }
+template <typename T, int N, int V, int L, int R1>
+__global__ void __launch_bounds__(L *(N / V), (lane_row_minb<N, V, L>())) k_lane_r2c(const RowArgs a) {
+    lane_r2c_tile<T, N, V, L, R1>(a, blockIdx.x);
+}
 
 // P5, lane per position: same arithmetic as k_fast_c2r
-template <typename T, int N, int V, int L, int R1>
-__global__ void __launch_bounds__(L *(N / V), (lane_row_minb<N, V, L>())) k_lane_c2r(const RowArgs a) {
+template <typename T, int N, int V, int L, int R1, bool COH>
+__device__ __forceinline__ void lane_c2r_tile(const RowArgs &a, unsigned bx) {
     using C = cx_t<T>;
     constexpr int TPL = N / V;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *buf = reinterpret_cast<C *>(smem_raw);
     const int tid = threadIdx.x, t = tid % TPL, l = tid / TPL;
-    const long long row = (long long)blockIdx.x * L + l;
+    const long long row = (long long)bx * L + l;
     const bool live = row < a.nrows;
     const C *crow = reinterpret_cast<const C *>(a.c) + (live ? row : 0) * row_pitch(N);
     C x[V];
 #pragma unroll
-    for (int c = 0; c < V; ++c) x[c] = live ? crow[t + c * TPL] : C{T(0), T(0)};
-    const C xn = live && t == 0 ? crow[N] : C{T(0), T(0)};
+    for (int c = 0; c < V; ++c) x[c] = live ? (COH ? ldcg_c(crow + t + c * TPL) : crow[t + c * TPL]) : C{T(0), T(0)};
+    const C xn = live && t == 0 ? (COH ? ldcg_c(crow + N) : crow[N]) : C{T(0), T(0)};
     // Z[q] = A + i conj(w^q) B, Z[N-q] = conj A + i w^q conj B for q <= N/2,
     // A, B from (X[q], X[N-q]).  Positions t + c TPL and t + (V-1-c) TPL are
     // done together: their partners are registers V-1-c and c of lane TPL - t
@@ -816,6 +829,10 @@ __global__ void __launch_bounds__(L *(N / V), (lane_row_minb<N, V, L>())) k_lane
 #pragma unroll
         for (int c = 0; c < V / 2; ++c) store_pair<T>(xr, t + c * TPL, v[c]);
     }
+}
+template <typename T, int N, int V, int L, int R1>
+__global__ void __launch_bounds__(L *(N / V), (lane_row_minb<N, V, L>())) k_lane_c2r(const RowArgs a) {
+    lane_c2r_tile<T, N, V, L, R1, false>(a, blockIdx.x);
 }
 
 // ----------------------------------------------------- configurations --
