@@ -226,8 +226,8 @@ def measured_peaks():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-KERNEL_SOURCES = ["fast.cuh", "fast_col_body.inc", "fast.h", "fast_f32.cu", "fast_f64.cu", "fast_df.cu", "df.cuh", "fft_engine.cuh",
-                  "kernels.cuh"]
+KERNEL_SOURCES = ["fast.cuh", "fast_col_body.inc", "fast.h", "fast_f32.cu", "fast_f64.cu", "fast_fx.cuh", "fx.cuh", "fx_line.cuh",
+                  "fft_engine.cuh", "kernels.cuh"]
 
 
 def kernel_src_sha():

@@ -56,21 +56,19 @@ typedef enum {
 /* The paper's solver names HOCKNEY, VICO and VICO_2 (Sec. 4, availability). */
 typedef enum { FSP_HE = 0, FSP_VG = 1, FSP_VG_DCT = 2 } fsp_algo;
 
-/* FSP_F64: every step in double precision.
+/* FSP_F64: double arrays, the transforms in 64-bit fixed point at a scale of
+ * each line's own (rounding at or below that of double-precision sums).
  * FSP_F32_MIXED: the solve (all transforms and the spectral multiply) in
  * single precision; the Green's spectrum is precomputed in double precision
  * and rounded once to single precision.
- * FSP_F64_DF: double arrays in and out, FP64-class accuracy (about 1e-14
- * relative), but the transforms run in double-float arithmetic (each value a
- * pair of floats, hi + lo) on the FP32 pipes, which on this GPU are far faster
- * than its FP64 pipes; the spectrum is the FP64 one split into float pairs.
- * Only where the specialised kernels run: N = 32, 64, 128, 256, 512, or a
- * non-cubic box whose sizes are powers of two in that range
- * (FSP_EUNSUPPORTED otherwise); not in batches.  Double-float keeps FP32's
- * exponent range: plan creation returns FSP_EUNSUPPORTED when the largest
- * spectrum value lies outside [2^-80, 2^80] (that value is about
- * 3e-6 L^2 (32/N)^3, so the box side L may range over about 1e-8 .. 1e14 at
- * N = 32 .. 512), and the caller keeps 8 N^3 max|rho| below about 2^80. */
+ * FSP_F64_DF: double arrays in and out at FP64-class accuracy; since the FP64
+ * passes run in 64-bit fixed point, which is faster and more accurate than the
+ * float pairs this type was made for, it is now the same solve as FSP_F64.
+ * Its limits stay: N = 32, 64, 128, 256, 512, or a non-cubic box whose sizes
+ * are powers of two in that range (FSP_EUNSUPPORTED otherwise); not in
+ * batches; plan creation returns FSP_EUNSUPPORTED when the largest spectrum
+ * value lies outside [2^-80, 2^80] (that value is about 3e-6 L^2 (32/N)^3, so
+ * the box side L may range over about 1e-8 .. 1e14 at N = 32 .. 512). */
 typedef enum { FSP_F64 = 0, FSP_F32_MIXED = 1, FSP_F64_DF = 2 } fsp_dtype;
 
 typedef struct fsp_plan fsp_plan;

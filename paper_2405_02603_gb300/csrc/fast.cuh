@@ -29,7 +29,6 @@
 #include <type_traits>
 #include <utility>
 
-#include "df.cuh"
 #include "fast.h"
 #include "fx.cuh"
 #include "kernels.cuh"
@@ -56,44 +55,16 @@ __host__ __device__ constexpr double cos32(int m) {
 }
 __host__ __device__ constexpr double sin32(int m) { return cos32(m - 8); }
 
-// Type of the caller's real arrays (rho, phi): the compute type itself, except
-// for double-float, whose solves read and write double.
-template <typename T> struct io_of {
-    using t = T;
-};
-template <> struct io_of<df> {
-    using t = double;
-};
-template <typename T> __device__ __forceinline__ cx_t<T> load_pair(const typename io_of<T>::t *row, int m) {
-    if constexpr (std::is_same<T, df>::value) {
-        const double2 q = reinterpret_cast<const double2 *>(row)[m];
-        return cdf{df_from_double(q.x), df_from_double(q.y)};
-    } else {
-        return reinterpret_cast<const cx_t<T> *>(row)[m];
-    }
+template <typename T> __device__ __forceinline__ cx_t<T> load_pair(const T *row, int m) {
+    return reinterpret_cast<const cx_t<T> *>(row)[m];
 }
-template <typename T> __device__ __forceinline__ void store_pair(typename io_of<T>::t *row, int m, cx_t<T> v) {
-    if constexpr (std::is_same<T, df>::value)
-        reinterpret_cast<double2 *>(row)[m] = double2{df_to_double(v.x), df_to_double(v.y)};
-    else
-        reinterpret_cast<cx_t<T> *>(row)[m] = v;
+template <typename T> __device__ __forceinline__ void store_pair(T *row, int m, cx_t<T> v) {
+    reinterpret_cast<cx_t<T> *>(row)[m] = v;
 }
 
 // loads that bypass L1 (ld.global.cg): streamed data and spectrum values
 // are read once per CTA, so they should not evict the twiddle table from L1
 __device__ __forceinline__ float2 ldcg_c(const float2 *p) { return __ldcg(p); }
-__device__ __forceinline__ double2 ldcg_c(const double2 *p) { return __ldcg(p); }
-__device__ __forceinline__ cdf ldcg_c(const cdf *p) {
-    const float4 q = __ldcg(reinterpret_cast<const float4 *>(p));
-    return cdf{df(q.x, q.y, 0), df(q.z, q.w, 0)};
-}
-__device__ __forceinline__ float ldcg_r(const float *p) { return __ldcg(p); }
-__device__ __forceinline__ double ldcg_r(const double *p) { return __ldcg(p); }
-__device__ __forceinline__ df ldcg_r(const df *p) {
-    const float2 q = __ldcg(reinterpret_cast<const float2 *>(p));
-    return df(q.x, q.y, 0);
-}
-
 template <int I, int E> struct StaticFor {
     template <class F> static __device__ __forceinline__ void run(F &&f) {
         if constexpr (I < E) {
@@ -441,15 +412,13 @@ template <int n, int MODE> struct ColGeo {
 // Per (type, pass) choices, each measured on the GB300 at N = 256:
 //   PF:  prefetch the thread's spectrum values into L1 before the forward
 //        transform (P3: their latency overlaps the transform; FP32 P3 -5 %).
-//   TWS: roots table in shared memory: double-float P3 -11 % and P2 -2 %,
-//        the FP32 field P3 (COL_FMO) and the FP32 P3 on lines of 1024 (-4 %)
-//        faster too; the FP32 P3 of the potential on lines of 512, native
-//        FP64 and every P4 are slower or unchanged with it.
+//   TWS: roots table in shared memory: the FP32 field P3 (COL_FMO) and the
+//        FP32 P3 on lines of 1024 (-4 %) are faster with it; the FP32 P3 of
+//        the potential on lines of 512 and every P4 slower or unchanged.
 template <typename T, int MODE, int n> struct ColOpt {
     static constexpr bool ZL = MODE == COL_FMI || MODE == COL_FMO;
-    static constexpr bool DF = std::is_same<T, df>::value;
     static constexpr bool F32 = std::is_same<T, float>::value;
-    static constexpr bool PF = ZL && !DF;
+    static constexpr bool PF = ZL;
     // CTAs per SM the register allocation must allow (2: k_fast_col_occ2):
     // two 256-thread tiles of the FP32 P3 on lines of 512 (N = 256)
     static constexpr int MINB = ZL && F32 && n == 512 ? 2 : 1;
@@ -465,8 +434,7 @@ template <typename T, int MODE, int n> struct ColOpt {
     // load at an immediate offset, no index arithmetic per twiddle
     // (measured: N = 256 P3 0.191 -> 0.183 ms; N = 128 2 % slower, so off there)
     static constexpr bool TT = MODE == COL_FMI && F32 && n == 512;
-    static constexpr bool TWS = (DF && MODE != COL_INV) || (MODE == COL_FMO && !std::is_same<T, double>::value) ||
-                                (MODE == COL_FMI && F32 && n == 1024);
+    static constexpr bool TWS = MODE == COL_FMO || (MODE == COL_FMI && F32 && n == 1024);
 };
 
 // RG (a non-cubic box): the strides, the number of lines (k_x <= n_x) and the
@@ -519,7 +487,7 @@ __device__ __forceinline__ void fast_r2c_tile(const RowArgs &a, unsigned bx) {
     C *buf = reinterpret_cast<C *>(smem_raw);
     const int tid = threadIdx.x, l = tid % L, t = tid / L;
     const long long row0 = (long long)bx * L;
-    using R = typename io_of<T>::t;
+    using R = T;
     const R *x = reinterpret_cast<const R *>(a.x);
     // coalesced row loads of the packed pairs (x[2m], x[2m+1]), m < N/2, all
     // of a thread's loads issued before the first shared-memory store
@@ -649,7 +617,7 @@ __device__ __forceinline__ void fast_c2r_tile(const RowArgs &a, unsigned bx) {
 #pragma unroll
         for (int r = 0; r < RL / 2; ++r) buf[(t + k * TPL + r * (N / RL)) * LD + l] = v[k * RL + r];
     __syncthreads();
-    using R = typename io_of<T>::t;
+    using R = T;
     R *x = reinterpret_cast<R *>(const_cast<void *>(a.x));
 #pragma unroll 4
     for (int idx = tid; idx < L * H; idx += NTH) {
@@ -728,7 +696,7 @@ __device__ __forceinline__ void lane_r2c_tile(const RowArgs &a, unsigned bx) {
     const int tid = threadIdx.x, t = tid % TPL, l = tid / TPL;
     const long long row = (long long)bx * L + l;
     const bool live = row < a.nrows;
-    using R = typename io_of<T>::t;
+    using R = T;
     const R *xr = reinterpret_cast<const R *>(a.x) + (live ? row : 0) * N;
     const C *tw = reinterpret_cast<const C *>(a.tw);
     C v[V];
@@ -823,7 +791,7 @@ __device__ __forceinline__ void lane_c2r_tile(const RowArgs &a, unsigned bx) {
     }
     lane_row_stages<T, +1, N, V, L, R1>(v, buf, t, l, reinterpret_cast<const C *>(a.tw), false, true);
     // the first N/2 positions t + c TPL (c < V/2) hold z[m] = (x[2m], x[2m+1])
-    using R = typename io_of<T>::t;
+    using R = T;
     R *xr = reinterpret_cast<R *>(const_cast<void *>(a.x)) + (live ? row : 0) * N;
     if (live) {
 #pragma unroll
@@ -862,12 +830,6 @@ FSP_CFG(float, 256, 16, 16, 16, 16, 1)
 FSP_CFG(float, 512, 32, 16, 16, 32, 1)
 FSP_CFG(float, 1024, 16, 16, 16, 16, 4)
 FSP_CFG(float, 2048, 16, 8, 16, 16, 8)  // column passes of non-cubic boxes only (an axis of 1024)
-FSP_CFG(df, 32, 8, 16, 4, 8, 1)
-FSP_CFG(df, 64, 8, 16, 8, 8, 1)
-FSP_CFG(df, 128, 16, 8, 8, 16, 1)
-FSP_CFG(df, 256, 8, 8, 8, 8, 4)
-FSP_CFG(df, 512, 8, 8, 8, 8, 8)
-FSP_CFG(df, 1024, 16, 8, 16, 8, 8)
 #undef FSP_CFG
 
 // A column pass may override its length's shape (each measured on the GB300):

@@ -1,6 +1,6 @@
 // fast_field.h -- host interface of the field's P3 on non-cubic boxes: the
 // odd-spectrum column pass (COL_FMO) with runtime geometry, instantiated with
-// the cubic field P3 in fast_{f32,f64,df}_field.cu.
+// the cubic field P3 in fast_{f32,f64}_field.cu.
 #pragma once
 #include <cuda_runtime.h>
 

@@ -7,7 +7,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "df.cuh"
 #include "greens.h"
 
 namespace fsp {
@@ -286,8 +285,6 @@ cudaError_t launch_vg_sample_full3(void *g, const int *n, const double *h, doubl
 }
 
 template cudaError_t launch_store_S<float>(const double *, void *, int, int, double, cudaStream_t);
-template cudaError_t launch_store_S<df>(const double *, void *, int, int, double, cudaStream_t);
-template cudaError_t launch_load_S<df>(const void *, double *, int, int, cudaStream_t);
 template cudaError_t launch_store_S<double>(const double *, void *, int, int, double, cudaStream_t);
 template cudaError_t launch_load_S<float>(const void *, double *, int, int, cudaStream_t);
 template cudaError_t launch_load_S<double>(const void *, double *, int, int, cudaStream_t);
@@ -295,7 +292,5 @@ template cudaError_t launch_store_S3<float>(const double *, void *, int, long lo
 template cudaError_t launch_store_S3<double>(const double *, void *, int, long long, int, double, cudaStream_t);
 template cudaError_t launch_load_S3<float>(const void *, double *, int, long long, int, cudaStream_t);
 template cudaError_t launch_load_S3<double>(const void *, double *, int, long long, int, cudaStream_t);
-template cudaError_t launch_store_S3<df>(const double *, void *, int, long long, int, double, cudaStream_t);
-template cudaError_t launch_load_S3<df>(const void *, double *, int, long long, int, cudaStream_t);
 
 }  // namespace fsp

@@ -76,7 +76,7 @@ __device__ __forceinline__ void discard_l2(const void *p) {
 // imaginary parts at k_x = 0.  Through the length-N FFT of the packed pairs
 // z[m] = x[2m] + i x[2m+1] (zero for m >= N/2, the padding).
 template <typename T, int N, int V, int L, int R1, int R2, int R3>
-__device__ __forceinline__ void plane_r2c_tile(const typename io_of<T>::t *x, cx_t<T> *w1, cx_t<T> *buf,
+__device__ __forceinline__ void plane_r2c_tile(const T *x, cx_t<T> *w1, cx_t<T> *buf,
                                                const cx_t<T> *tw, const cx_t<T> *tw2) {
     using C = cx_t<T>;
     constexpr int TPL = N / V, LD = L + 1, NTH = L * TPL, H = N / 2, P = row_pitch(N);
@@ -137,7 +137,7 @@ __device__ __forceinline__ void plane_r2c_tile(const typename io_of<T>::t *x, cx
 // L rows of packed half spectra (W1) -> the first N of the 2N real outputs.
 // The W1 lines are read through L2 only and discarded after use.
 template <typename T, int N, int V, int L, int R1, int R2, int R3>
-__device__ __forceinline__ void plane_c2r_tile(cx_t<T> *w1, typename io_of<T>::t *x, cx_t<T> *buf,
+__device__ __forceinline__ void plane_c2r_tile(cx_t<T> *w1, T *x, cx_t<T> *buf,
                                                const cx_t<T> *tw, const cx_t<T> *tw2) {
     using C = cx_t<T>;
     constexpr int TPL = N / V, LD = L + 1, NTH = L * TPL, H = N / 2, P = row_pitch(N);
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(PlaneGeo<T, N>::NTH, PlaneCfg<T, N>::MINB) k_p
     using K = PlaneCfg<T, N>;
     using G = PlaneGeo<T, N>;
     using C = cx_t<T>;
-    using R = typename io_of<T>::t;
+    using R = T;
     constexpr int n = G::n, P = G::P;
     extern __shared__ __align__(16) unsigned char plane_smem[];
     C *buf = reinterpret_cast<C *>(plane_smem);
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(PlaneGeo<T, N>::NTH, PlaneCfg<T, N>::MINB) k_p
     using K = PlaneCfg<T, N>;
     using G = PlaneGeo<T, N>;
     using C = cx_t<T>;
-    using R = typename io_of<T>::t;
+    using R = T;
     constexpr int n = G::n, P = G::P;
     extern __shared__ __align__(16) unsigned char plane_smem[];
     C *buf = reinterpret_cast<C *>(plane_smem);
