@@ -121,8 +121,11 @@ template <bool COH, typename V> __device__ __forceinline__ V ldw(const V *p) {
         return *p;
 }
 
+// whether a complex line carries two real ones
+__host__ __device__ constexpr bool lines_pair(int in) { return in != IN_CPLX; }
+
 // ---------------------------------------------------------- lines_tile --
-// One tile of a batched line transform: lines [bx*L, bx*L + L) of batch `by`.
+// One tile of a batched line transform: (complex) lines [bx*L, bx*L + L) of batch `by`.
 // Every thread of the CTA must call it (barriers); threads beyond L*tpl idle.
 template <typename T, int IN, int OUT, int MODE, bool COH>
 __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long by, unsigned char *smem_raw) {
@@ -130,6 +133,8 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
     using C = cx_t<W>;
     using IC = cx_t<T>;
     constexpr bool FX = std::is_same<W, fx>::value;
+    constexpr bool PAIR = lines_pair(IN);
+    static_assert(!PAIR || OUT == OUT_REAL, "pairs of real lines have real transforms");
     __shared__ TileLines tl;
     if constexpr (FX) tile_clear(tl);
     C *buf = reinterpret_cast<C *>(smem_raw);
@@ -186,6 +191,9 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
         // y[2M - j] = x[j] for 0 < j < M.  DST-I through the DFT of
         // y[j] = i x[j], y[2M - j] = -i x[j] for 0 < j < M, y[0] = y[M] = 0,
         // which is 2 sum_j x[j] sin(pi j k / M), real.
+        //
+        // A complex line holds two real ones (2 c and 2 c + 1, as its real and
+        // imaginary part): both transforms are real, so they come out apart.
         const T *in = reinterpret_cast<const T *>(a.in) + b * a.in_batch;
         const int M = n >> 1, np = M + 1, cnt = L * np;
         const bool col = (a.in_line == 1);
@@ -198,22 +206,25 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
                 p = idx % np;
                 l = idx / np;
             }
-            T x = T(0);
-            if (line0 + l < a.nlines) x = ldw<COH>(in + ((long long)(line0 + l) * a.in_line + (long long)p * a.in_pos));
+            const int r0 = 2 * (line0 + l);
+            const T *q = in + ((long long)r0 * a.in_line + (long long)p * a.in_pos);
+            T x = T(0), y = T(0);
+            if (r0 < a.nlines) x = ldw<COH>(q);
+            if (r0 + 1 < a.nlines) y = ldw<COH>(q + a.in_line);
             const bool inner = p > 0 && p < M;
             if (IN == IN_REAL_EVEN) {
-                buf[p * ld + l] = C{tile_real(x), W(0)};
-                if (inner) buf[(n - p) * ld + l] = C{tile_real(x), W(0)};
-            } else {
-                buf[p * ld + l] = C{W(0), tile_real(inner ? x : T(0))};
-                if (inner) buf[(n - p) * ld + l] = C{W(0), tile_real(-x)};
+                buf[p * ld + l] = C{tile_real(x), tile_real(y)};
+                if (inner) buf[(n - p) * ld + l] = C{tile_real(x), tile_real(y)};
+            } else {  // i (x + i y)
+                buf[p * ld + l] = inner ? C{tile_real(-y), tile_real(x)} : C{W(0), W(0)};
+                if (inner) buf[(n - p) * ld + l] = C{tile_real(y), tile_real(-x)};
             }
         }
     }
     __syncthreads();
 
     const int l = tid & lmask, sub = tid >> a.lgL;
-    const bool act = (line0 + l) < a.nlines && sub < a.tpl;
+    const bool act = (PAIR ? 2 * (line0 + l) : line0 + l) < a.nlines && sub < a.tpl;
     const fx_tw_t<W> *tw = reinterpret_cast<const fx_tw_t<W> *>(a.tw);
     FxScale sc{};
     if constexpr (FX) {
@@ -318,8 +329,17 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
                 p = idx % a.n_out;
                 ll = idx / a.n_out;
             }
-            if (line0 + ll < a.nlines)
+            if constexpr (PAIR) {
+                const int r0 = 2 * (line0 + ll);
+                if (r0 < a.nlines) {
+                    const IC v = tile_out(buf[p * ld + ll], tl, ll);
+                    T *q = out + ((long long)r0 * a.out_line + (long long)p * a.out_pos);
+                    q[0] = v.x;
+                    if (r0 + 1 < a.nlines) q[a.out_line] = v.y;
+                }
+            } else if (line0 + ll < a.nlines) {
                 out[(long long)(line0 + ll) * a.out_line + (long long)p * a.out_pos] = tile_out_re(buf[p * ld + ll], tl, ll);
+            }
         }
     }
 }
@@ -548,7 +568,8 @@ template <typename T, int IN, int OUT, int MODE> cudaError_t launch_lines(const 
     auto kern = k_lines<T, IN, OUT, MODE>;
     cudaError_t e = set_smem(kern, sm);
     if (e != cudaSuccess) return e;
-    dim3 grid((unsigned)((a.nlines + (1 << a.lgL) - 1) >> a.lgL), (unsigned)a.nbatch);
+    const int nl = lines_pair(IN) ? (a.nlines + 1) / 2 : a.nlines;
+    dim3 grid((unsigned)((nl + (1 << a.lgL) - 1) >> a.lgL), (unsigned)a.nbatch);
     kern<<<grid, (1 << a.lgL) * a.tpl, sm, s>>>(a);
     return cudaGetLastError();
 }
