@@ -32,6 +32,7 @@
 #include "fast.h"
 #include "fx.cuh"
 #include "kernels.cuh"
+#include "pdl.cuh"
 
 namespace fsp {
 namespace fast {
@@ -452,15 +453,18 @@ __device__ __forceinline__ void fast_col_body(const ColArgs &a, unsigned bx, uns
 }
 template <typename T, int n, int V, int L, int R1, int R2, int R3, int MODE, bool RG = false>
 __global__ void __launch_bounds__(L *(n / V)) k_fast_col(const ColArgs a) {
+    pdl_wait();
     const unsigned bx = blockIdx.x, by = blockIdx.y;
 #include "fast_col_body.inc"
 }
 template <typename T, int n, int V, int L, int R1, int R2, int R3, int MODE, bool RG = false>
 __global__ void __launch_bounds__(L *(n / V), 2) k_fast_col_occ2(const ColArgs a) {
+    pdl_wait();
     fast_col_body<T, n, V, L, R1, R2, R3, MODE, RG>(a, blockIdx.x, blockIdx.y);
 }
 template <typename T, int n, int V, int L, int R1, int R2, int R3, int MODE, bool RG = false>
 __global__ void __launch_bounds__(L *(n / V)) k_fast_col_inl(const ColArgs a) {
+    pdl_wait();
     fast_col_body<T, n, V, L, R1, R2, R3, MODE, RG>(a, blockIdx.x, blockIdx.y);
 }
 template <typename T, int n, int V, int L, int R1, int R2, int R3, int MODE, bool RG>
@@ -551,6 +555,7 @@ __device__ __forceinline__ void fast_r2c_tile(const RowArgs &a, unsigned bx) {
 }
 template <typename T, int N, int V, int L, int R1, int R2, int R3>
 __global__ void __launch_bounds__(L *(N / V)) k_fast_r2c(const RowArgs a) {
+    pdl_wait();
     fast_r2c_tile<T, N, V, L, R1, R2, R3>(a, blockIdx.x);
 }
 
@@ -627,6 +632,7 @@ __device__ __forceinline__ void fast_c2r_tile(const RowArgs &a, unsigned bx) {
 }
 template <typename T, int N, int V, int L, int R1, int R2, int R3>
 __global__ void __launch_bounds__(L *(N / V)) k_fast_c2r(const RowArgs a) {
+    pdl_wait();
     fast_c2r_tile<T, N, V, L, R1, R2, R3, false>(a, blockIdx.x);
 }
 
@@ -736,6 +742,7 @@ __device__ __forceinline__ void lane_r2c_tile(const RowArgs &a, unsigned bx) {
 }
 template <typename T, int N, int V, int L, int R1>
 __global__ void __launch_bounds__(L *(N / V), (lane_row_minb<N, V, L>())) k_lane_r2c(const RowArgs a) {
+    pdl_wait();
     lane_r2c_tile<T, N, V, L, R1>(a, blockIdx.x);
 }
 
@@ -800,6 +807,7 @@ __device__ __forceinline__ void lane_c2r_tile(const RowArgs &a, unsigned bx) {
 }
 template <typename T, int N, int V, int L, int R1>
 __global__ void __launch_bounds__(L *(N / V), (lane_row_minb<N, V, L>())) k_lane_c2r(const RowArgs a) {
+    pdl_wait();
     lane_c2r_tile<T, N, V, L, R1, false>(a, blockIdx.x);
 }
 
@@ -907,8 +915,7 @@ template <typename T, int n, int MODE> cudaError_t launch_col_n(const ColArgs &a
         static_assert(N % K::L == 0, "tiles must cover k_x < N exactly");
         if (nbatch % N != 0) return cudaErrorInvalidValue;
         dim3 grid((unsigned)(N / K::L), (unsigned)(nbatch + nbatch / N));
-        kern<<<grid, K::L * (n / K::V), sm, s>>>(a);
-        return cudaGetLastError();
+        return launch_pass(kern, grid, K::L * (n / K::V), sm, s, a);
     }
 }
 
@@ -929,8 +936,7 @@ template <typename T, int n, int MODE> cudaError_t launch_col_rg_n(const ColArgs
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
         dim3 grid((unsigned)(nx / K::L), (unsigned)(nbatch + b.xrows));
-        kern<<<grid, K::L * (n / K::V), sm, s>>>(b);
-        return cudaGetLastError();
+        return launch_pass(kern, grid, K::L * (n / K::V), sm, s, b);
     }
 }
 
@@ -964,8 +970,8 @@ template <typename T, int N, bool R2C> cudaError_t launch_row_n(const RowArgs &a
         }
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
-        kern<<<(unsigned)((a.nrows + K::L - 1) / K::L), K::L * (N / K::V), sm, s>>>(a);
-        return cudaGetLastError();
+        const dim3 grid((unsigned)((a.nrows + K::L - 1) / K::L));
+        return launch_pass(kern, grid, K::L * (N / K::V), sm, s, a);
     }
 }
 

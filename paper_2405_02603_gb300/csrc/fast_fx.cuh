@@ -112,6 +112,7 @@ __device__ __forceinline__ void fx_rest(cfx *v, cfx *buf, int t, int l, const fx
 // Column passes: tiles, geometry and Nyquist blocks as in fast_col_body.inc.
 template <int n, int V, int L, int R1, int R2, int R3, int MODE, bool RG, int MINB>
 __global__ void __launch_bounds__(L *(n / V), MINB) k_fx_col(const ColArgs a) {
+    pdl_wait();
     using G = ColGeo<n, MODE>;
     constexpr int TPL = n / V, N = G::N, NTH = L * TPL;
     constexpr int RL = LastR<R1, R2, R3>::value, NT = R3 > 1 ? 2 : 1;
@@ -241,6 +242,7 @@ __global__ void __launch_bounds__(L *(n / V), MINB) k_fx_col(const ColArgs a) {
 // P1: k_fast_r2c in fixed point.
 template <int N, int V, int L, int R1, int R2, int R3>
 __global__ void __launch_bounds__(L *(N / V)) k_fx_r2c(const RowArgs a) {
+    pdl_wait();
     constexpr int TPL = N / V, LD = L + 1, NTH = L * TPL, H = N / 2;
     constexpr int RL = LastR<R1, R2, R3>::value, NT = R3 > 1 ? 2 : 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -326,6 +328,7 @@ __global__ void __launch_bounds__(L *(N / V)) k_fx_r2c(const RowArgs a) {
 // P5: k_fast_c2r in fixed point.
 template <int N, int V, int L, int R1, int R2, int R3>
 __global__ void __launch_bounds__(L *(N / V)) k_fx_c2r(const RowArgs a) {
+    pdl_wait();
     constexpr int TPL = N / V, LD = L + 1, NTH = L * TPL, H = N / 2;
     constexpr int RL = LastR<R1, R2, R3>::value, NT = R3 > 1 ? 2 : 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -470,8 +473,7 @@ template <int n, int MODE, bool RG> cudaError_t launch_fx_col_n(const ColArgs &a
             b.xrows = (nbatch / K::L + nx / K::L - 1) / (nx / K::L);
             grid = dim3((unsigned)(nx / K::L), (unsigned)(nbatch + b.xrows));
         }
-        kern<<<grid, K::L * (n / K::V), sm, s>>>(b);
-        return cudaGetLastError();
+        return launch_pass(kern, grid, K::L * (n / K::V), sm, s, b);
     }
 }
 template <int MODE> cudaError_t launch_fx_col(int n, const ColArgs &a, int nbatch, cudaStream_t s) {
@@ -504,8 +506,8 @@ template <int N, bool R2C> cudaError_t launch_fx_row_n(const RowArgs &a, cudaStr
     const size_t sm = sizeof(cfx) * (N + 1) * (K::L + 1);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)((a.nrows + K::L - 1) / K::L), K::L * (N / K::V), sm, s>>>(a);
-    return cudaGetLastError();
+    const dim3 grid((unsigned)((a.nrows + K::L - 1) / K::L));
+    return launch_pass(kern, grid, K::L * (N / K::V), sm, s, a);
 }
 template <bool R2C> cudaError_t launch_fx_row(int N, const RowArgs &a, cudaStream_t s) {
     switch (N) {

@@ -347,6 +347,7 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
 template <typename T, int IN, int OUT, int MODE>
 __global__ void __launch_bounds__(kMaxThreads) k_lines(const LinesArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_wait();
     lines_tile<T, IN, OUT, MODE, false>(a, blockIdx.x, blockIdx.y, smem_raw);
 }
 
@@ -444,6 +445,7 @@ __device__ __forceinline__ void r2c_tile(const RowsArgs &a, int bx, unsigned cha
 
 template <typename T> __global__ void __launch_bounds__(kMaxThreads) k_r2c_rows(const RowsArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_wait();
     r2c_tile<T, false>(a, blockIdx.x, smem_raw);
 }
 
@@ -535,6 +537,7 @@ __device__ __forceinline__ void c2r_tile(const RowsArgs &a, int bx, unsigned cha
 
 template <typename T> __global__ void __launch_bounds__(kMaxThreads) k_c2r_rows(const RowsArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_wait();
     c2r_tile<T, false>(a, blockIdx.x, smem_raw);
 }
 
@@ -570,24 +573,23 @@ template <typename T, int IN, int OUT, int MODE> cudaError_t launch_lines(const 
     if (e != cudaSuccess) return e;
     const int nl = lines_pair(IN) ? (a.nlines + 1) / 2 : a.nlines;
     dim3 grid((unsigned)((nl + (1 << a.lgL) - 1) >> a.lgL), (unsigned)a.nbatch);
-    kern<<<grid, (1 << a.lgL) * a.tpl, sm, s>>>(a);
-    return cudaGetLastError();
+    return launch_pass(kern, grid, (1 << a.lgL) * a.tpl, sm, s, a);
 }
 
 template <typename T> cudaError_t launch_r2c_rows(const RowsArgs &a, cudaStream_t s) {
     const size_t sm = rows_smem_bytes<T>(a);
     cudaError_t e = set_smem(k_r2c_rows<T>, sm);
     if (e != cudaSuccess) return e;
-    k_r2c_rows<T><<<(unsigned)((a.nrows + (1 << a.lgL) - 1) >> a.lgL), (1 << a.lgL) * a.tpl, sm, s>>>(a);
-    return cudaGetLastError();
+    const dim3 grid((unsigned)((a.nrows + (1 << a.lgL) - 1) >> a.lgL));
+    return launch_pass(k_r2c_rows<T>, grid, (1 << a.lgL) * a.tpl, sm, s, a);
 }
 
 template <typename T> cudaError_t launch_c2r_rows(const RowsArgs &a, cudaStream_t s) {
     const size_t sm = rows_smem_bytes<T>(a);
     cudaError_t e = set_smem(k_c2r_rows<T>, sm);
     if (e != cudaSuccess) return e;
-    k_c2r_rows<T><<<(unsigned)((a.nrows + (1 << a.lgL) - 1) >> a.lgL), (1 << a.lgL) * a.tpl, sm, s>>>(a);
-    return cudaGetLastError();
+    const dim3 grid((unsigned)((a.nrows + (1 << a.lgL) - 1) >> a.lgL));
+    return launch_pass(k_c2r_rows<T>, grid, (1 << a.lgL) * a.tpl, sm, s, a);
 }
 
 template <typename T> cudaError_t launch_roots(void *tw, int n, cudaStream_t s) {

@@ -325,6 +325,7 @@ __global__ void __launch_bounds__(PlaneGeo<T, N>::NTH, PlaneCfg<T, N>::MINB) k_p
     using R = T;
     constexpr int n = G::n, P = G::P;
     extern __shared__ __align__(16) unsigned char plane_smem[];
+    pdl_wait();
     C *buf = reinterpret_cast<C *>(plane_smem);
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const int c = (int)cluster.block_rank();
@@ -357,6 +358,7 @@ __global__ void __launch_bounds__(PlaneGeo<T, N>::NTH, PlaneCfg<T, N>::MINB) k_p
     using R = T;
     constexpr int n = G::n, P = G::P;
     extern __shared__ __align__(16) unsigned char plane_smem[];
+    pdl_wait();
     C *buf = reinterpret_cast<C *>(plane_smem);
     cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
     const int c = (int)cluster.block_rank();

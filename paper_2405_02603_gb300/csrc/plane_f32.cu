@@ -17,13 +17,14 @@ template <typename T, int N> cudaError_t launch_plane_n(bool fwd, const PlaneArg
     cfg.blockDim = dim3((unsigned)G::NTH);
     cfg.dynamicSmemBytes = G::SMEM;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = K::C;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    at[1] = pdl_attribute();
+    cfg.numAttrs = 2;
     e = cudaLaunchKernelEx(&cfg, kern, a);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
