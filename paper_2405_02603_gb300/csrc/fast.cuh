@@ -265,6 +265,25 @@ template <typename T, int D, bool PK = false> struct RD {
         v[1] = add(e[1], o1), v[4] = sub(e[1], o1);
         v[2] = add(e[2], o2), v[5] = sub(e[2], o2);
     }
+    // Radix 12 = 3 x 4 without twiddles (Good-Thomas): inputs 4 n1 + 3 n2,
+    // outputs 4 k1 + 9 k2, both mod 12.
+    template <bool HZ, bool HO> static __device__ __forceinline__ void d12(C *v) {
+        static_assert(!HZ && !HO, "radix 12 runs only as a middle stage");
+        C y[12];
+#pragma unroll
+        for (int n2 = 0; n2 < 4; ++n2) {
+            C g[3] = {v[(3 * n2) % 12], v[(4 + 3 * n2) % 12], v[(8 + 3 * n2) % 12]};
+            d3<false, false>(g);
+#pragma unroll
+            for (int k1 = 0; k1 < 3; ++k1) y[k1 * 4 + n2] = g[k1];
+        }
+#pragma unroll
+        for (int k1 = 0; k1 < 3; ++k1) {
+            d4<false, false>(y + k1 * 4);
+#pragma unroll
+            for (int k2 = 0; k2 < 4; ++k2) v[(4 * k1 + 9 * k2) % 12] = y[k1 * 4 + k2];
+        }
+    }
     template <int R, bool HZ, bool HO> static __device__ __forceinline__ void dft(C *v) {
         if constexpr (R == 2)
             d2<HZ, HO>(v);
@@ -278,6 +297,8 @@ template <typename T, int D, bool PK = false> struct RD {
             d6<HZ, HO>(v);
         else if constexpr (R == 8)
             d8<HZ, HO>(v);
+        else if constexpr (R == 12)
+            d12<HZ, HO>(v);
         else
             dct4<R, HZ, HO>(v);
     }

@@ -88,10 +88,57 @@ template <int D, int n, int V, int L> struct Fst {
     }
 };
 
+// The exchanges between stages.  With 8 or more lines a quarter warp (what
+// shared memory serves at once, 8 lanes of 16 bytes) stays within one
+// position and the pitch L + 1 does.  With 4 lines it covers two positions of
+// consecutive threads: a pitch of 5 would make every access a two-way
+// conflict, so the pitch is 4 and a position's lowest bit is flipped where
+// bits 3 and 4 differ, which puts positions 8 or 16 apart (the first stage's
+// stores) into different halves of a 128-byte row and leaves neighbours
+// there.  The flip depends on t and compile-time constants alone, so the
+// offsets of a thread's accesses stay immediates.  FP64 N = 256 1.95 -> 1.90
+// ms, N = 512 18.8 -> 18.0.
+template <int n, int V, int L> struct Fxc : Stg<fx, +1, n, V, L> {
+    static constexpr size_t smem = sizeof(cfx) * n * (L + 1);
+};
+template <int n, int V> struct Fxc<n, V, 4> {
+    static constexpr int TPL = n / V;
+    static constexpr size_t smem = sizeof(cfx) * n * 4;
+    static_assert(TPL % 32 == 0, "t alone decides the flips");
+    template <int R, int Ns> static __device__ __forceinline__ void store_out(cfx *buf, const cfx *v, int t, int l) {
+        static_assert((Ns == 1 && (R == 8 || R == 16)) || (R == 8 && (Ns == 8 || Ns == 16)), "flips worked out for these");
+        // position (t + k TPL - j) R + j + r Ns, j = t mod Ns; the flip is g,
+        // for odd h(r) 1 - g, with h a constant of r
+        const int j = t % Ns;
+        const int g = Ns == 1 ? (R == 8 ? (t ^ (t >> 1)) & 1 : t & 1) : Ns == 16 ? (j >> 3) & 1 : 0;
+        const int at = ((t - j) * R + j) * 4 + l;
+        StaticFor<0, V / R>::run([&](auto kc) {
+            constexpr int k = decltype(kc)::value;
+            StaticFor<0, R>::run([&](auto rc) {
+                constexpr int r = decltype(rc)::value, c = k * TPL * R + r * Ns;
+                constexpr int h = Ns == 1 ? (r >> 3) & 1 : Ns == 16 ? r & 1 : (r ^ (r >> 1)) & 1;
+                const int f = h ? 1 - g : g;
+                if constexpr (Ns == 1)  // the lowest bit of the position is r's
+                    buf[at + c * 4 + (r & 1 ? -4 * f : 4 * f)] = v[k * R + r];
+                else  // ... is j's
+                    buf[(at ^ (f * 4)) + c * 4] = v[k * R + r];
+            });
+        });
+    }
+    template <int R> static __device__ __forceinline__ void load_in(cfx *v, const cfx *buf, int t, int l) {
+        static_assert((n / R) % 32 == 0, "t alone decides the flip");
+        const cfx *b = buf + ((t ^ (((t >> 3) ^ (t >> 4)) & 1)) * 4 + l);
+#pragma unroll
+        for (int k = 0; k < V / R; ++k)
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[k * R + r] = b[(k * TPL + r * (n / R)) * 4];
+    }
+};
+
 // stages 1.. of the schedule after stage 0 in registers (run_rest of fast.cuh)
 template <int D, int n, int V, int L, int R1, int R2, int R3, bool HO_LAST>
 __device__ __forceinline__ void fx_rest(cfx *v, cfx *buf, int t, int l, const fxw *tw, bool first_sync) {
-    using X = Stg<fx, D, n, V, L>;  // its exchanges
+    using X = Fxc<n, V, L>;
     using F = Fst<D, n, V, L>;
     if (first_sync) __syncthreads();
     X::template store_out<R1, 1>(buf, v, t, l);
@@ -409,7 +456,8 @@ __global__ void __launch_bounds__(L *(N / V)) k_fx_c2r(const RowArgs a) {
 // Tile shape and radix schedule per length: V values per thread, L lines.
 // Measured at N = 256 (lines of 512), per pass: 8*8*8 with 4 lines (256
 // threads) 0.28 ms for P2 and P4 and 1.07 for P3, with 8 lines 0.31 / 0.32 /
-// 1.13, 16*16*2 with V = 16 0.30 / 0.30 / 1.10.
+// 1.13, 16*16*2 with V = 16 0.30 / 0.30 / 1.10 (before the exchanges of 4 lines
+// were free of conflicts).
 template <int n> struct CfgX {
     static constexpr bool Ok = false;
     static constexpr int V = 8, L = 8, R1 = 8, R2 = 8, R3 = 1;
@@ -426,7 +474,7 @@ FSP_CFGX(32, 4, 8, 4, 2, 4)
 FSP_CFGX(64, 4, 8, 4, 4, 4)
 FSP_CFGX(96, 12, 8, 4, 6, 4)
 FSP_CFGX(128, 8, 8, 8, 2, 8)
-FSP_CFGX(192, 24, 8, 8, 3, 8)
+FSP_CFGX(192, 12, 8, 4, 12, 4)
 FSP_CFGX(256, 8, 8, 8, 4, 8)
 FSP_CFGX(384, 24, 8, 8, 6, 8)
 FSP_CFGX(512, 8, 4, 8, 8, 8)
@@ -441,13 +489,14 @@ template <> struct RowX<64> {
 template <> struct RowX<256> {
     static constexpr int V = 16, L = 8, R1 = 16, R2 = 16, R3 = 1;
 };
-// CTAs per SM the registers must allow: 32 warps for P3 with V = 8 (64
-// registers: a few spill, and it is still the fastest: 1.07 ms at N = 256
-// against 1.08 with 24 warps and 1.19 with 16), 16 with V = 16
+// CTAs per SM the registers must allow.  With 8 values per thread 24 warps for
+// P3 (80 registers, a few spilled: 1.055 ms at N = 256, 1.063 with 32 warps,
+// 1.14 with 16) and 32 for P2 and P4 (0.266 / 0.255 ms, 0.273 / 0.274 with
+// 24); fewer where a thread holds more.
 template <int n, int MODE> constexpr int fx_minb() {
     constexpr int th = CfgX<n>::L * (n / CfgX<n>::V), V = CfgX<n>::V;
-    if (MODE != COL_FMI && MODE != COL_FMO) return 1;
-    return V <= 8 ? 1024 / th : V <= 16 ? 512 / th : 1;
+    if (MODE != COL_FMI && MODE != COL_FMO) return V <= 8 ? 1024 / th : 1;
+    return V <= 8 ? 768 / th : V <= 12 ? 640 / th : V <= 16 ? 512 / th : 1;
 }
 
 template <int n, int MODE, bool RG> cudaError_t launch_fx_col_n(const ColArgs &a, int nbatch, cudaStream_t s) {
@@ -456,7 +505,7 @@ template <int n, int MODE, bool RG> cudaError_t launch_fx_col_n(const ColArgs &a
         return cudaErrorInvalidValue;
     } else {
         auto kern = k_fx_col<n, K::V, K::L, K::R1, K::R2, K::R3, MODE, RG, fx_minb<n, MODE>()>;
-        const size_t sm = sizeof(cfx) * n * (K::L + 1);
+        const size_t sm = Fxc<n, K::V, K::L>::smem;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
         if (e != cudaSuccess) return e;
         ColArgs b = a;
