@@ -441,16 +441,17 @@ template <typename T, int MODE, int n> struct ColOpt {
     static constexpr bool ZL = MODE == COL_FMI || MODE == COL_FMO;
     static constexpr bool F32 = std::is_same<T, float>::value;
     static constexpr bool PF = ZL;
-    // CTAs per SM the register allocation must allow (2: k_fast_col_occ2):
-    // two 256-thread tiles of the FP32 P3 on lines of 512 (N = 256)
-    static constexpr int MINB = ZL && F32 && n == 512 ? 2 : 1;
+    // CTAs per SM the register allocation aims at (2: k_fast_col_occ2): P3 on
+    // lines of 512 (N = 256), which the compiler would take to one, and P2 on
+    // lines of 512 and 1024, which it would take to three
+    static constexpr int MINB = F32 && ((ZL && n == 512) || (MODE == COL_FWD && (n == 512 || n == 1024))) ? 2 : 1;
     // PK: packed two-float complex sums in the register DFTs, on the FP32
     // lines of 512 of P3 (0.206 -> 0.191 ms) and P2 (0.090 -> 0.084 ms);
     // P4 unchanged by them, the lines of 1024 6-8 % slower, so off there
     static constexpr bool PK = F32 && n == 512 && (ZL || MODE == COL_FWD);
-    // INL: k_fast_col_inl for the FP32 P2 on lines of 512 (0.084 ms against
-    // 0.088 with the body in the kernel)
-    static constexpr bool INL = F32 && n == 512 && MODE == COL_FWD;
+    // INL: k_fast_col_inl for the cubic P3 on lines of 1024 (1.95 ms against
+    // 2.10 with the body in the kernel)
+    static constexpr bool INL = F32 && n == 1024 && MODE == COL_FMI;
     // TT: the twiddled stages of the cubic P3 read per-stage tables [j][r]
     // (after the n roots; see p3_table_fill): a pair of twiddles per 16-byte
     // load at an immediate offset, no index arithmetic per twiddle
@@ -492,7 +493,7 @@ template <typename T, int n, int V, int L, int R1, int R2, int R3, int MODE, boo
 constexpr auto col_kernel() {
     if constexpr (ColOpt<T, MODE, n>::MINB == 2)
         return k_fast_col_occ2<T, n, V, L, R1, R2, R3, MODE, RG>;
-    else if constexpr (ColOpt<T, MODE, n>::INL)
+    else if constexpr (ColOpt<T, MODE, n>::INL && !RG)
         return k_fast_col_inl<T, n, V, L, R1, R2, R3, MODE, RG>;
     else
         return k_fast_col<T, n, V, L, R1, R2, R3, MODE, RG>;
@@ -861,15 +862,21 @@ FSP_CFG(float, 1024, 16, 16, 16, 16, 4)
 FSP_CFG(float, 2048, 16, 8, 16, 16, 8)  // column passes of non-cubic boxes only (an axis of 1024)
 #undef FSP_CFG
 
-// A column pass may override its length's shape (each measured on the GB300):
-// at n = 1024 the FP32 inverse-only pass (P4) is faster with V = 32, L = 8,
-// 32*32 (0.66 vs 0.80 ms at N = 512), the passes with a forward transform with
-// V = 16, L = 16, 16*16*4; at n = 512 P4 is faster with V = 16, L = 16,
-// 16*16*2 (0.078 vs 0.092 ms at N = 256), P2 and P3 with V = 32, L = 16, 16*32.
+// A column pass may override its length's shape (each measured on the GB300).
+// N = 512, lines of 1024: P2 32*32 with 8 lines 0.63 ms (16*16*4 with 16 lines
+// 0.79), P3 32*32 with 16 lines 1.95 (16*16*4 2.22), P4 32*32 with 8 lines 0.65
+// (16*16*4 0.82).  N = 256, lines of 512: P2 16*32 0.072 ms (16*16*2 0.083), P4
+// 16*16*2 0.075 (16*32 0.088).  The two-stage P2 shapes are held to two CTAs per
+// SM (ColOpt::MINB): with three the shared memory leaves the L1 too small for
+// the roots (lines of 1024 0.83 ms instead of 0.63).
 template <typename T, int n, int MODE> struct ColCfg : Cfg<T, n> {};
 template <> struct ColCfg<float, 1024, COL_INV> {
     static constexpr bool Ok = true;
     static constexpr int V = 32, L = 8, R1 = 32, R2 = 32, R3 = 1;
+};
+template <> struct ColCfg<float, 1024, COL_FMI> {
+    static constexpr bool Ok = true;
+    static constexpr int V = 32, L = 16, R1 = 32, R2 = 32, R3 = 1;
 };
 template <> struct ColCfg<float, 512, COL_INV> {
     static constexpr bool Ok = true;
@@ -877,8 +884,16 @@ template <> struct ColCfg<float, 512, COL_INV> {
 };
 template <> struct ColCfg<float, 512, COL_FWD> {
     static constexpr bool Ok = true;
-    static constexpr int V = 16, L = 16, R1 = 16, R2 = 16, R3 = 2;
+    static constexpr int V = 32, L = 16, R1 = 16, R2 = 32, R3 = 1;
 };
+template <> struct ColCfg<float, 1024, COL_FWD> {
+    static constexpr bool Ok = true;
+    static constexpr int V = 32, L = 8, R1 = 32, R2 = 32, R3 = 1;
+};
+// non-cubic boxes (runtime strides): the cube's shapes, but for P3 on lines of
+// 1024 (256 x 256 x 512: 0.565 ms with 16*16*4, 0.582 with 32*32)
+template <typename T, int n, int MODE> struct ColCfgRG : ColCfg<T, n, MODE> {};
+template <> struct ColCfgRG<float, 1024, COL_FMI> : Cfg<float, 1024> {};
 
 template <typename T, int n> constexpr size_t smem_for(int positions) {
     return (size_t)positions * (Cfg<T, n>::L + 1) * sizeof(cx_t<T>);
@@ -943,7 +958,7 @@ template <typename T, int n, int MODE> cudaError_t launch_col_n(const ColArgs &a
 // Non-cubic box: lines k_x <= n_x = nlines - 1 (a multiple of L), nbatch a
 // multiple of L; ceil(nbatch / n_x) leading block rows hold the Nyquist tiles.
 template <typename T, int n, int MODE> cudaError_t launch_col_rg_n(const ColArgs &a, int nbatch, cudaStream_t s) {
-    using K = ColCfg<T, n, MODE>;
+    using K = ColCfgRG<T, n, MODE>;
     if constexpr (!K::Ok) {
         return cudaErrorInvalidValue;
     } else {
