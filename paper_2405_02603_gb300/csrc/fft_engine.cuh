@@ -79,6 +79,15 @@ template <int B, int E> struct Unroll {
     }
 };
 
+// Quotients and remainders by a number known once per kernel or stage: one
+// division, then a multiply each (x d < 2^32).
+struct FastDiv {
+    unsigned m;
+    int d;
+    __device__ __forceinline__ explicit FastDiv(int dd) : m(dd > 1 ? 0xffffffffu / (unsigned)dd + 1u : 0u), d(dd) {}
+    __device__ __forceinline__ int quot(int x) const { return d > 1 ? (int)__umulhi((unsigned)x, m) : x; }
+};
+
 // Radix schedule of a length-n transform, always in the order: n5 radix-5
 // stages, n3 radix-3 stages, n8 radix-8 stages, then one radix-`last` stage
 // (last = 4, 2 or 0 for none).  A fixed order keeps each radix in its own
@@ -207,12 +216,13 @@ template <typename T, int D> struct Engine {
             }
         });
         __syncthreads();
-        const int tws = n / (Ns * R);
+        const FastDiv by_ns(Ns), by_r(Ns * R);
+        const int tws = by_r.quot(n);
         Unroll<0, KMAX>::run([&](auto kc) {
             constexpr int k = decltype(kc)::value;
             const int b = sub + k * tpl;
             if (act && b < nb) {
-                const int j = b % Ns;
+                const int j = b - by_ns.quot(b) * Ns;
                 // fixed point: every stage but the first divides by 4
                 if (std::is_same<TW, C>::value ? j != 0 : Ns > 1) {
                     if constexpr (!std::is_same<TW, C>::value) v[k * R] = tw_of<T>::quarter(v[k * R]);

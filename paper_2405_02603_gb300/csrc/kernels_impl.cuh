@@ -14,6 +14,10 @@
 namespace fsp {
 
 constexpr int kMaxThreads = 512;
+// 512-thread CTAs per SM the registers must allow: two in FP32 (64 registers;
+// left to itself the compiler takes 72-74 for some passes: N = 225 1.47 ms
+// instead of 1.27), one in fixed point
+template <typename T> constexpr int lines_minb() { return sizeof(T) == 4 ? 2 : 1; }
 constexpr int kMaxLines = 32;  // lines per CTA (lgL <= 5)
 
 template <typename T> struct work_of {
@@ -168,11 +172,12 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
                 }
             }
         } else {
+            const FastDiv by(a.n_in);
             for (int base = tid; base < cnt; base += U * nth) {
                 C q[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int idx = base + u * nth, p = idx % a.n_in, l = idx / a.n_in;
+                    const int idx = base + u * nth, l = by.quot(idx), p = idx - l * a.n_in;
                     q[u] = C{W(0), W(0)};
                     if (idx < cnt && line0 + l < a.nlines)
                         q[u] = tile_cplx(ldw<COH>(in + ((long long)(line0 + l) * a.in_line + (long long)p * a.in_pos)));
@@ -180,7 +185,8 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int idx = base + u * nth;
-                    if (idx < cnt) buf[(idx % a.n_in) * ld + idx / a.n_in] = q[u];
+                    const int l = by.quot(idx);
+                    if (idx < cnt) buf[(idx - l * a.n_in) * ld + l] = q[u];
                 }
             }
         }
@@ -197,14 +203,15 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
         const T *in = reinterpret_cast<const T *>(a.in) + b * a.in_batch;
         const int M = n >> 1, np = M + 1, cnt = L * np;
         const bool col = (a.in_line == 1);
+        const FastDiv by(np);
         for (int idx = tid; idx < cnt; idx += nth) {
             int l, p;
             if (col) {
                 l = idx & lmask;
                 p = idx >> a.lgL;
             } else {
-                p = idx % np;
-                l = idx / np;
+                l = by.quot(idx);
+                p = idx - l * np;
             }
             const int r0 = 2 * (line0 + l);
             const T *q = in + ((long long)r0 * a.in_line + (long long)p * a.in_pos);
@@ -304,6 +311,7 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
     // ---- store (crop to n_out positions)
     const int cnt = L * a.n_out;
     const bool col = (a.out_line == 1);
+    const FastDiv by_out(a.n_out);
     if (OUT == OUT_CPLX) {
         IC *out = reinterpret_cast<IC *>(a.out) + b * a.out_batch;
         for (int idx = tid; idx < cnt; idx += nth) {
@@ -312,8 +320,8 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
                 ll = idx & lmask;
                 p = idx >> a.lgL;
             } else {
-                p = idx % a.n_out;
-                ll = idx / a.n_out;
+                ll = by_out.quot(idx);
+                p = idx - ll * a.n_out;
             }
             if (line0 + ll < a.nlines)
                 out[(long long)(line0 + ll) * a.out_line + (long long)p * a.out_pos] = tile_out(buf[p * ld + ll], tl, ll);
@@ -326,8 +334,8 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
                 ll = idx & lmask;
                 p = idx >> a.lgL;
             } else {
-                p = idx % a.n_out;
-                ll = idx / a.n_out;
+                ll = by_out.quot(idx);
+                p = idx - ll * a.n_out;
             }
             if constexpr (PAIR) {
                 const int r0 = 2 * (line0 + ll);
@@ -345,7 +353,7 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
 }
 
 template <typename T, int IN, int OUT, int MODE>
-__global__ void __launch_bounds__(kMaxThreads) k_lines(const LinesArgs a) {
+__global__ void __launch_bounds__(kMaxThreads, lines_minb<T>()) k_lines(const LinesArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_wait();
     lines_tile<T, IN, OUT, MODE, false>(a, blockIdx.x, blockIdx.y, smem_raw);
@@ -373,12 +381,13 @@ __device__ __forceinline__ void r2c_tile(const RowsArgs &a, int bx, unsigned cha
     const T *x = reinterpret_cast<const T *>(a.x);
 
     const int cnt = L * Mh;
+    const FastDiv by(Mh);
     constexpr int U = 4;  // loads in flight per thread
     for (int base = tid; base < cnt; base += U * nth) {
         C q[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int idx = base + u * nth, m = idx % Mh, l = idx / Mh;
+            const int idx = base + u * nth, l = by.quot(idx), m = idx - l * Mh;
             q[u] = C{W(0), W(0)};
             if (idx < cnt && row0 + l < a.nrows) {
                 const T *xr = x + (row0 + l) * a.x_row;
@@ -393,7 +402,8 @@ __device__ __forceinline__ void r2c_tile(const RowsArgs &a, int bx, unsigned cha
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int idx = base + u * nth;
-            if (idx < cnt) buf[(idx % Mh) * ld + idx / Mh] = q[u];
+            const int l = by.quot(idx);
+            if (idx < cnt) buf[(idx - l * Mh) * ld + l] = q[u];
         }
     }
     const int zc = L * (N - Mh);
@@ -437,13 +447,14 @@ __device__ __forceinline__ void r2c_tile(const RowsArgs &a, int bx, unsigned cha
 
     IC *c = reinterpret_cast<IC *>(a.c);
     const int np = N + 1, cnt2 = L * np;
+    const FastDiv by_np(np);
     for (int idx = tid; idx < cnt2; idx += nth) {
-        const int k = idx % np, ll = idx / np;
+        const int ll = by_np.quot(idx), k = idx - ll * np;
         if (row0 + ll < a.nrows) c[(row0 + ll) * a.c_row + k] = tile_out(buf[k * ld + ll], tl, ll);
     }
 }
 
-template <typename T> __global__ void __launch_bounds__(kMaxThreads) k_r2c_rows(const RowsArgs a) {
+template <typename T> __global__ void __launch_bounds__(kMaxThreads, lines_minb<T>()) k_r2c_rows(const RowsArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_wait();
     r2c_tile<T, false>(a, blockIdx.x, smem_raw);
@@ -471,19 +482,21 @@ __device__ __forceinline__ void c2r_tile(const RowsArgs &a, int bx, unsigned cha
     const IC *c = reinterpret_cast<const IC *>(a.c);
 
     const int cnt = L * np;
+    const FastDiv by(np);
     constexpr int U = 4;  // loads in flight per thread
     for (int base = tid; base < cnt; base += U * nth) {
         C q[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int idx = base + u * nth, k = idx % np, l = idx / np;
+            const int idx = base + u * nth, l = by.quot(idx), k = idx - l * np;
             q[u] = C{W(0), W(0)};
             if (idx < cnt && row0 + l < a.nrows) q[u] = tile_cplx(ldw<COH>(c + ((row0 + l) * a.c_row + k)));
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int idx = base + u * nth;
-            if (idx < cnt) buf[(idx % np) * ld + idx / np] = q[u];
+            const int l = by.quot(idx);
+            if (idx < cnt) buf[(idx - l * np) * ld + l] = q[u];
         }
     }
     __syncthreads();
@@ -520,8 +533,9 @@ __device__ __forceinline__ void c2r_tile(const RowsArgs &a, int bx, unsigned cha
 
     T *x = reinterpret_cast<T *>(const_cast<void *>(a.x));
     const int Mh = (N + 1) >> 1, cnt2 = L * Mh;
+    const FastDiv by_m(Mh);
     for (int idx = tid; idx < cnt2; idx += nth) {
-        const int m = idx % Mh, ll = idx / Mh;
+        const int ll = by_m.quot(idx), m = idx - ll * Mh;
         if (row0 + ll < a.nrows) {
             T *xr = x + (row0 + ll) * a.x_row;
             const IC v = tile_out(buf[m * ld + ll], tl, ll);
@@ -535,7 +549,7 @@ __device__ __forceinline__ void c2r_tile(const RowsArgs &a, int bx, unsigned cha
     }
 }
 
-template <typename T> __global__ void __launch_bounds__(kMaxThreads) k_c2r_rows(const RowsArgs a) {
+template <typename T> __global__ void __launch_bounds__(kMaxThreads, lines_minb<T>()) k_c2r_rows(const RowsArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     pdl_wait();
     c2r_tile<T, false>(a, blockIdx.x, smem_raw);
