@@ -99,6 +99,14 @@ template <typename T, int D, bool PK = false> struct RD {
             return csub(a, b);
     }
 
+    // a / 2 (fixed point: a shift instead of a product)
+    static __device__ __forceinline__ T halve(T a) {
+        if constexpr (std::is_same<T, fx>::value)
+            return fx_halve(a);
+        else
+            return T(0.5) * a;
+    }
+
     // multiply by exp(D 2 pi i M / 32)
     template <int M> static __device__ __forceinline__ C w32(C a) {
         constexpr int m = ((M % 32) + 32) % 32;
@@ -226,7 +234,7 @@ template <typename T, int D, bool PK = false> struct RD {
         static_assert(!HZ && !HO, "radix 3 runs only as a middle stage");
         constexpr T s3 = T(D * 0.86602540378443864676372317075294);
         const C a = v[0], t = add(v[1], v[2]), d = sub(v[1], v[2]);
-        const C u = C{a.x - T(0.5) * t.x, a.y - T(0.5) * t.y};
+        const C u = C{a.x - halve(t.x), a.y - halve(t.y)};
         const C w = C{-s3 * d.y, s3 * d.x};
         v[0] = add(a, t);
         v[1] = add(u, w);
@@ -237,6 +245,10 @@ template <typename T, int D, bool PK = false> struct RD {
     // c1 t2 +- i D (s2 t3 - s1 t4); c_k = cos(2 pi k / 5), s_k = sin(2 pi k / 5).
     template <bool HZ, bool HO> static __device__ __forceinline__ void d5(C *v) {
         static_assert(!HZ && !HO, "radix 5 runs only as a middle stage");
+        if constexpr (std::is_same<T, fx>::value) {
+            d5_few(v);
+            return;
+        }
         constexpr T c1 = T(0.30901699437494742410229341718282), c2 = T(-0.80901699437494742410229341718282);
         constexpr T s1 = T(D * 0.95105651629515357211643933337938), s2 = T(D * 0.58778525229247312916870595463907);
         const C v0 = v[0], t1 = add(v[1], v[4]), t2 = add(v[2], v[3]), t3 = sub(v[1], v[4]),
@@ -251,6 +263,27 @@ template <typename T, int D, bool PK = false> struct RD {
         v[2] = C{m2.x - n2.y, m2.y + n2.x};
         v[3] = C{m2.x + n2.y, m2.y - n2.x};
     }
+    // The same with 8 products instead of 16, for fixed point, whose products
+    // cost several sums: c1 t1 + c2 t2 = -(t1 + t2)/4 + (sqrt 5 / 4)(t1 - t2),
+    // and with p = s2 (t3 + t4), s1 t3 + s2 t4 = p + (s1 - s2) t3, s2 t3 - s1 t4 =
+    // p - (s1 + s2) t4.
+    static __device__ __forceinline__ void d5_few(C *v) {
+        constexpr T r5 = T(0.55901699437494742410229341718282), s2 = T(D * 0.58778525229247312916870595463907);
+        constexpr T sd = T(D * 0.36327126400268044294773337874031);   // s1 - s2
+        constexpr T sh = T(D * 0.76942088429381335752825644667730);   // (s1 + s2) / 2
+        const C v0 = v[0], t1 = add(v[1], v[4]), t2 = add(v[2], v[3]), t3 = sub(v[1], v[4]), t4 = sub(v[2], v[3]);
+        const C ts = add(t1, t2), td = sub(t1, t2), tt = add(t3, t4);
+        const C q = C{v0.x - fx_quarter(ts.x), v0.y - fx_quarter(ts.y)}, e = C{r5 * td.x, r5 * td.y};
+        const C m1 = add(q, e), m2 = sub(q, e);
+        const C p = C{s2 * tt.x, s2 * tt.y};
+        const C n1 = C{p.x + sd * t3.x, p.y + sd * t3.y};
+        const C n2 = C{p.x - sh * (t4.x + t4.x), p.y - sh * (t4.y + t4.y)};
+        v[0] = add(v0, ts);
+        v[1] = C{m1.x - n1.y, m1.y + n1.x};
+        v[4] = C{m1.x + n1.y, m1.y - n1.x};
+        v[2] = C{m2.x - n2.y, m2.y + n2.x};
+        v[3] = C{m2.x + n2.y, m2.y - n2.x};
+    }
     // Radix 6 = 2 x 3: E = DFT3 of the even inputs, O of the odd ones,
     // X[q] = E[q] + w6^q O[q], X[q+3] = E[q] - w6^q O[q], w6 = exp(D 2 pi i / 6).
     template <bool HZ, bool HO> static __device__ __forceinline__ void d6(C *v) {
@@ -259,8 +292,8 @@ template <typename T, int D, bool PK = false> struct RD {
         C e[3] = {v[0], v[2], v[4]}, o[3] = {v[1], v[3], v[5]};
         d3<false, false>(e);
         d3<false, false>(o);
-        const C o1 = C{T(0.5) * o[1].x - s3 * o[1].y, s3 * o[1].x + T(0.5) * o[1].y};    // w6 o1
-        const C o2 = C{-T(0.5) * o[2].x - s3 * o[2].y, s3 * o[2].x - T(0.5) * o[2].y};   // w6^2 o2
+        const C o1 = C{halve(o[1].x) - s3 * o[1].y, s3 * o[1].x + halve(o[1].y)};      // w6 o1
+        const C o2 = C{-halve(o[2].x) - s3 * o[2].y, s3 * o[2].x - halve(o[2].y)};     // w6^2 o2
         v[0] = add(e[0], o[0]), v[3] = sub(e[0], o[0]);
         v[1] = add(e[1], o1), v[4] = sub(e[1], o1);
         v[2] = add(e[2], o2), v[5] = sub(e[2], o2);

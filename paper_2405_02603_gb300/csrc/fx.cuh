@@ -85,6 +85,8 @@ template <int D> __device__ __forceinline__ cfx fx_twiddle(cfx x, fxw w) {
     return fx_cmul(x.x.v, x.y.v, w.rh, w.rl, -w.ih, -w.il, w.ih, w.il);
 }
 __device__ __forceinline__ fx fx_quarter(fx a) { return fx((a.v + 2) >> 2, 0); }
+// a / 2
+__device__ __forceinline__ fx fx_halve(fx a) { return fx((a.v + 1) >> 1, 0); }
 // as the generic engine calls them
 template <> struct tw_of<fx> {
     using t = fxw;
