@@ -99,6 +99,15 @@ template <typename T, int D, bool PK = false> struct RD {
             return csub(a, b);
     }
 
+    // a constant: c, or in fixed point its 63 fraction bits
+    static __device__ __forceinline__ constexpr T cst(double c, long long q63) {
+        if constexpr (std::is_same<T, fx>::value)
+            return fx(q63, 0);
+        else
+            return T(c);
+    }
+    static constexpr double kSin60 = 0.86602540378443864676372317075294;
+    static constexpr long long kSin60Q = 7987674492471257551LL;
     // a / 2 (fixed point: a shift instead of a product)
     static __device__ __forceinline__ T halve(T a) {
         if constexpr (std::is_same<T, fx>::value)
@@ -232,7 +241,7 @@ template <typename T, int D, bool PK = false> struct RD {
     // padded first or a cropped last stage (those stay even).
     template <bool HZ, bool HO> static __device__ __forceinline__ void d3(C *v) {
         static_assert(!HZ && !HO, "radix 3 runs only as a middle stage");
-        constexpr T s3 = T(D * 0.86602540378443864676372317075294);
+        constexpr T s3 = cst(D * kSin60, D * kSin60Q);
         const C a = v[0], t = add(v[1], v[2]), d = sub(v[1], v[2]);
         const C u = C{a.x - halve(t.x), a.y - halve(t.y)};
         const C w = C{-s3 * d.y, s3 * d.x};
@@ -267,10 +276,11 @@ template <typename T, int D, bool PK = false> struct RD {
     // cost several sums: c1 t1 + c2 t2 = -(t1 + t2)/4 + (sqrt 5 / 4)(t1 - t2),
     // and with p = s2 (t3 + t4), s1 t3 + s2 t4 = p + (s1 - s2) t3, s2 t3 - s1 t4 =
     // p - (s1 + s2) t4.
+    // (Constants with 63 fraction bits.)
     static __device__ __forceinline__ void d5_few(C *v) {
-        constexpr T r5 = T(0.55901699437494742410229341718282), s2 = T(D * 0.58778525229247312916870595463907);
-        constexpr T sd = T(D * 0.36327126400268044294773337874031);   // s1 - s2
-        constexpr T sh = T(D * 0.76942088429381335752825644667730);   // (s1 + s2) / 2
+        constexpr T r5 = T(5156021714044493573LL, 0), s2 = T(D * 5421362059670026167LL, 0);
+        constexpr T sd = T(D * 3350586018195211715LL, 0);  // s1 - s2
+        constexpr T sh = T(D * 7096655068767632024LL, 0);  // (s1 + s2) / 2
         const C v0 = v[0], t1 = add(v[1], v[4]), t2 = add(v[2], v[3]), t3 = sub(v[1], v[4]), t4 = sub(v[2], v[3]);
         const C ts = add(t1, t2), td = sub(t1, t2), tt = add(t3, t4);
         const C q = C{v0.x - fx_quarter(ts.x), v0.y - fx_quarter(ts.y)}, e = C{r5 * td.x, r5 * td.y};
@@ -288,7 +298,7 @@ template <typename T, int D, bool PK = false> struct RD {
     // X[q] = E[q] + w6^q O[q], X[q+3] = E[q] - w6^q O[q], w6 = exp(D 2 pi i / 6).
     template <bool HZ, bool HO> static __device__ __forceinline__ void d6(C *v) {
         static_assert(!HZ && !HO, "radix 6 runs only as a middle stage");
-        constexpr T s3 = T(D * 0.86602540378443864676372317075294);
+        constexpr T s3 = cst(D * kSin60, D * kSin60Q);
         C e[3] = {v[0], v[2], v[4]}, o[3] = {v[1], v[3], v[5]};
         d3<false, false>(e);
         d3<false, false>(o);
