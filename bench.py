@@ -42,7 +42,6 @@ import fsp_inputs as I  # noqa: E402
 
 METRIC = "VG free-space solves/s at N=256 (FP32-mix vs FP64, stated err); HBM GB/s; p99 ms"
 FALLBACK_HBM_GBS = 6800.0
-FP64_PEAK_TFLOPS = 1.25  # nominal dense FP64 rate of a GB300
 PASS_NAMES = ["P1 pad + x-R2C (k_fast_r2c)", "P2 y-FFT (k_fast_col fwd)", "P3 z-FFT * S * z-IFFT (k_fast_col fmi)",
               "P4 y-IFFT (k_fast_col inv)", "P5 x-C2R + crop (k_fast_c2r)"]
 NSRC = 4
@@ -101,7 +100,7 @@ def profile_case(args):
     print(json.dumps({"profile_case": args.profile_case, "N": N, "ok": True, "launches_per_solve": cases}))
 
 
-PASS_KERNELS = ("k_fast_", "k_lane_", "k_plane_", "k_p3_tma")  # the solve passes of the profile cases (N = 256)
+PASS_KERNELS = ("k_fast_", "k_lane_", "k_plane_", "k_p3_tma", "k_fx_")  # the solve passes of the profile cases (N = 256)
 
 
 def read_ncu_csv(path):
@@ -495,7 +494,8 @@ def roofline(N, c, r, leg, dtype, hbm, hbm_kind):
     k = int(np.argmax(share))
     dur_s = float(leg["per_pass"][:, k].mean()) * 1e-3
     achieved = pb[k] / dur_s / 1e9
-    return {"bound": "hbm", "kernel": PASS_NAMES[k], "achieved": round(achieved, 1), "peak": hbm,
+    name = PASS_NAMES[k] if dtype == "f32" else PASS_NAMES[k].replace("k_fast", "k_fx")
+    return {"bound": "hbm", "kernel": name, "achieved": round(achieved, 1), "peak": hbm,
             "unit": "GB/s", "frac": round(achieved / hbm, 4), "peak_kind": hbm_kind + " copy bandwidth",
             "traffic": recorded_traffic(dtype, N, k), "algorithmic_bytes": int(pb[k]),
             "pass_ms": [round(float(x), 4) for x in leg["per_pass"].mean(axis=0)],
@@ -543,7 +543,8 @@ def batch_leg(fsp, dtype, count=64, launches=5):
            "launches": launches}
     out.update(res[0])
     out["form"] = "one persistent kernel per launch over all 64 solves, CUDA graph replay"
-    out["tiles"] = "generic-engine tile shapes from the autotuned table paper_2405_02603_gb300/tuning/gb300.txt"
+    out["tiles"] = ("specialised passes in 128-thread tiles" if dtype == "f32" else
+                    "generic-engine tile shapes from the autotuned table paper_2405_02603_gb300/tuning/gb300.txt")
     out["graph_of_solves"] = dict(res[1], form="one CUDA graph of the 64 solves' own launches (the "
                                                "specialised kernels of every size in FP32; FP64: all but "
                                                "N = 160) on 8 streams")
@@ -755,7 +756,7 @@ def e2e_leg(fsp, plan, host_src, dtype, K, W):
 def precision_leg(fsp, Ns, L, W, world, with_oracle):
     """The precision configuration at the sizes other than the bench's N:
     VG-DCT solves of the seeded mixture (float32-rounded) in FP32-mixed, FP64
-    and double-float, each timed (solves/s) and compared with the oracle: the
+    and FSP_F64_DF, each timed (solves/s) and compared with the oracle: the
     whole field at N <= 256, at N = 512 the oracle's direct sum at 24 sampled
     points (its full FFT solve takes minutes there) and the whole field
     against this GPU's FP64 result."""
@@ -997,12 +998,8 @@ def main():
                    "hbm_gbs_solve": round(sum(pass_bytes(N, 16, 8)) / (t64 * 1e-3) / 1e9, 1),
                    "roofline": roofline(N, 16, 8, f64, "f64", hbm, hbm_kind),
                    "nominal_gflops": round(solve_flops(N) / (t64 * 1e-3) / 1e9, 1),
-                   "roofline_alu": {"bound": "alu", "achieved": round(solve_flops(N) / (t64 * 1e-3) / 1e12, 4),
-                                    "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                                    "frac": round(solve_flops(N) / (t64 * 1e-3) / 1e12 / FP64_PEAK_TFLOPS, 4),
-                                    "peak_kind": "nominal GB300 FP64 rate (a probe kernel measured 1.20)",
-                                    "flops": "nominal 5 n log2 n per complex FFT of length n, pruned work counted "
-                                             "as full"},
+                   "arithmetic": "64-bit fixed point at a scale per line, on the integer units; double arrays in "
+                                 "and out",
                    "precompute_ms": round(f64["precompute_ms"], 1), "gpu_launches": f64["launches"] * f64["K"]}
     tdf = fdf["tmax_ms"] / fdf["K"]
     out["fp64_df"] = {"value": round(fdf["value"], 2), "unit": "solves/s", "steps": fdf["K"], "ms_per_step": round(tdf, 4),
@@ -1010,7 +1007,7 @@ def main():
                       "p99_ms": round(float(np.percentile(fdf["per_step"], 99)), 4),
                       "hbm_gbs_solve": round(sum(pass_bytes(N, 16, 8)) / (tdf * 1e-3) / 1e9, 1),
                       "roofline": roofline(N, 16, 8, fdf, "f64df", hbm, hbm_kind),
-                      "arithmetic": "double-float (float pairs) on the FP32 pipes, double arrays in and out",
+                      "arithmetic": "the FP64 passes (64-bit fixed point), double arrays in and out",
                       "gpu_launches": fdf["launches"] * fdf["K"]}
     out["field"] = field_leg(fsp, N, L, args.algo, max(10, K // 4), W, world)
     out["field"]["roofline"].update({"peak": hbm, "frac": round(out["field"]["roofline"]["achieved"] / hbm, 4),
@@ -1039,7 +1036,6 @@ def main():
     # short scalar keys for the record (the objects above hold the details)
     out["fp64_value"] = out["fp64"]["value"]
     out["fp64_hbm_frac"] = out["fp64"]["roofline"]["frac"]
-    out["fp64_alu_frac"] = out["fp64"]["roofline_alu"]["frac"]
     out["fp64_df_value"] = out["fp64_df"]["value"]
     out["fp64_df_hbm_frac"] = out["fp64_df"]["roofline"]["frac"]
     out["e2e_value"] = f32["e2e"]["value"]

@@ -1219,7 +1219,7 @@ fsp_status fsp_plan_create_aniso(fsp_plan **out, int nx, int ny, int nz, double 
         fast_ok = fast_ok && ny >= 32 && nz >= 32;
         if (dtype != FSP_F64_DF) fast_ok = fast_ok && !generic_only;
     }
-    if (dtype == FSP_F64_DF && !fast_ok) return FSP_EUNSUPPORTED;  // double-float: specialised kernels only
+    if (dtype == FSP_F64_DF && !fast_ok) return FSP_EUNSUPPORTED;  // no generic engine for this type
     if (algo != FSP_HE) {
         // the (4 n_a h_a) periodisation of the truncated kernel must not reach
         // the box: 3 min_a L_a >= L_t = alpha |(L_x, L_y, L_z)|

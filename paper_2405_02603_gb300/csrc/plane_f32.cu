@@ -41,8 +41,8 @@ template <typename T> cudaError_t launch_plane(bool fwd, int N, const PlaneArgs 
 }  // namespace
 
 template <> bool has_plane<float>(int N) { return N == 64 || N == 128 || N == 256; }
-// N = 64: 0.0246 vs 0.0343 ms per solve.  N = 128 (0.068 vs 0.065) and N = 256
-// (0.506 vs 0.463): the plane passes are latency bound (one cluster barrier
+// N = 64: 0.0173 vs 0.0206 ms per solve.  N = 128 (0.063 vs 0.052) and N = 256
+// (0.477 vs 0.404): the plane passes are latency bound (one cluster barrier
 // per plane, 8 waves of 36 clusters at N = 256) and lose although W1 no
 // longer reaches HBM; they stay available for the A/B (FSP_PLANE=1).
 template <> bool plane_default<float>(int N) { return N == 64; }
