@@ -164,6 +164,17 @@ struct DevPool {
 std::mutex g_pool_mu;
 std::map<int, DevPool> g_pools;
 std::unordered_map<const void *, DevPool> g_pooled;  // live buffers of the pools
+std::vector<std::pair<void *, DevPool>> g_unsynced;  // freed while the device could not be waited for
+
+// While a StreamScope lives, what this thread frees was used on its stream
+// alone (plan-time temporaries), so a free waits for that stream and not for
+// the device: a plan can be made while another thread captures a graph.
+thread_local const cudaStream_t *t_free_stream = nullptr;
+struct StreamScope {
+    const cudaStream_t s, *prev;
+    explicit StreamScope(cudaStream_t st) : s(st), prev(t_free_stream) { t_free_stream = &s; }
+    ~StreamScope() { t_free_stream = prev; }
+};
 
 // the current device's pool (pool == nullptr: none could be made)
 DevPool dev_pool() {
@@ -196,7 +207,11 @@ cudaError_t plain_malloc(void **p, size_t bytes) {
         cudaError_t e = cudaMallocFromPoolAsync(p, bytes, d.pool, d.stream);
         if (e == cudaSuccess) {
             // usable on every stream from here on
-            if ((e = cudaStreamSynchronize(d.stream)) != cudaSuccess) return e;
+            if ((e = cudaStreamSynchronize(d.stream)) != cudaSuccess) {
+                cudaFreeAsync(*p, d.stream);
+                *p = nullptr;
+                return e;
+            }
             std::lock_guard<std::mutex> lk(g_pool_mu);
             g_pooled[*p] = d;
             return cudaSuccess;
@@ -206,14 +221,16 @@ cudaError_t plain_malloc(void **p, size_t bytes) {
     cudaError_t e = cudaMalloc(p, bytes);
     if (e == cudaErrorMemoryAllocation && d.pool) {
         cudaGetLastError();
-        cudaDeviceSynchronize();
+        cudaStreamSynchronize(d.stream);
         cudaMemPoolTrimTo(d.pool, 0);
         e = cudaMalloc(p, bytes);
     }
     return e;
 }
 
-// As cudaFree: everything enqueued on the device before is complete.
+// As cudaFree: everything enqueued on the device before is complete.  Where
+// waiting is refused (a stream in capture) the buffer is kept until a later
+// free can wait: another plan must not get memory that is still in use.
 void plain_free(void *p) {
     DevPool d;
     {
@@ -228,8 +245,16 @@ void plain_free(void *p) {
         cudaFree(p);
         return;
     }
-    cudaDeviceSynchronize();
-    cudaFreeAsync(p, d.stream);
+    if (t_free_stream && cudaStreamSynchronize(*t_free_stream) == cudaSuccess) {
+        cudaFreeAsync(p, d.stream);
+        return;
+    }
+    const bool idle = !t_free_stream && cudaDeviceSynchronize() == cudaSuccess;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    g_unsynced.emplace_back(p, d);
+    if (!idle) return;
+    for (const auto &q : g_unsynced) cudaFreeAsync(q.first, q.second.stream);
+    g_unsynced.clear();
 }
 
 void dev_free(void *p) {
@@ -1052,6 +1077,7 @@ fsp_status plan_create_impl(fsp_plan **out, int N, double L, double h, fsp_algo 
     fsp_plan *p = new fsp_plan();
     p->guarded = bounds_check_requested();
     GuardScope guard_scope(p->guarded);
+    StreamScope stream_scope(s);
     p->N = N, p->L = L, p->h = L / N, p->algo = algo, p->dtype = dtype;
     p->rsize = dtype == FSP_F32_MIXED ? 4 : 8;  // caller's reals
     p->P = ((N + 1) + 15) / 16 * 16;
@@ -1232,6 +1258,7 @@ fsp_status fsp_plan_create_aniso(fsp_plan **out, int nx, int ny, int nz, double 
     fsp_plan *p = new fsp_plan();
     p->guarded = bounds_check_requested();
     GuardScope guard_scope(p->guarded);
+    StreamScope stream_scope(s);
     p->aniso = true;
     p->fast = fast_ok;
     for (int a = 0; a < 3; ++a) p->n3[a] = nn[a], p->h3[a] = hh[a];
@@ -1332,6 +1359,7 @@ fsp_status fsp_plan_field_init(fsp_plan *plan, fsp_stream stream) {
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const auto t0 = std::chrono::steady_clock::now();
     GuardScope guard_scope(plan->guarded);
+    StreamScope stream_scope(s);
     const int N = plan->N;
     // the box: cubic, or the plan's non-cubic sizes and spacings
     const int nn[3] = {plan->aniso ? plan->n3[0] : N, plan->aniso ? plan->n3[1] : N, plan->aniso ? plan->n3[2] : N};
@@ -1577,6 +1605,7 @@ double fsp_plan_precompute_ms(const fsp_plan *plan) { return plan_live(plan) ? p
 
 fsp_status fsp_plan_spectrum(const fsp_plan *plan, double *s_host) {
     if (!plan_live(plan) || !s_host) return FSP_EINVAL;
+    StreamScope stream_scope(nullptr);
     if (plan->aniso) {
         const int kx = plan->n3[0] + 1;
         const long long rows = (long long)(plan->n3[1] + 1) * (plan->n3[2] + 1);
@@ -1604,6 +1633,7 @@ fsp_status fsp_kernel_T(int N, double L, fsp_algo algo, double *t_dev, fsp_strea
     if (st != FSP_OK) return st;
     if (!t_dev || !aligned16(t_dev)) return FSP_EINVAL;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    StreamScope stream_scope(s);
     Temps tmp;
     st = enqueue_kernel_T(N, L, algo, t_dev, s, tmp);
     cudaError_t e = cudaStreamSynchronize(s);
