@@ -275,19 +275,21 @@ template <typename T, int D, bool PK = false> struct RD {
     // The same with 8 products instead of 16, for fixed point, whose products
     // cost several sums: c1 t1 + c2 t2 = -(t1 + t2)/4 + (sqrt 5 / 4)(t1 - t2),
     // and with p = s2 (t3 + t4), s1 t3 + s2 t4 = p + (s1 - s2) t3, s2 t3 - s1 t4 =
-    // p - (s1 + s2) t4.
+    // p - t4 - (s1 + s2 - 1) t4: every step a sum of inputs times factors of
+    // modulus <= 1, which is what the line's scale leaves room for.
     // (Constants with 63 fraction bits.)
     static __device__ __forceinline__ void d5_few(C *v) {
         constexpr T r5 = T(5156021714044493573LL, 0), s2 = T(D * 5421362059670026167LL, 0);
         constexpr T sd = T(D * 3350586018195211715LL, 0);  // s1 - s2
-        constexpr T sh = T(D * 7096655068767632024LL, 0);  // (s1 + s2) / 2
+        constexpr T sh = T(D * 4969938100680488240LL, 0);  // s1 + s2 - 1
         const C v0 = v[0], t1 = add(v[1], v[4]), t2 = add(v[2], v[3]), t3 = sub(v[1], v[4]), t4 = sub(v[2], v[3]);
         const C ts = add(t1, t2), td = sub(t1, t2), tt = add(t3, t4);
         const C q = C{v0.x - fx_quarter(ts.x), v0.y - fx_quarter(ts.y)}, e = C{r5 * td.x, r5 * td.y};
         const C m1 = add(q, e), m2 = sub(q, e);
         const C p = C{s2 * tt.x, s2 * tt.y};
         const C n1 = C{p.x + sd * t3.x, p.y + sd * t3.y};
-        const C n2 = C{p.x - sh * (t4.x + t4.x), p.y - sh * (t4.y + t4.y)};
+        const C n2 = D > 0 ? C{p.x - t4.x - sh * t4.x, p.y - t4.y - sh * t4.y}
+                           : C{p.x + t4.x - sh * t4.x, p.y + t4.y - sh * t4.y};
         v[0] = add(v0, ts);
         v[1] = C{m1.x - n1.y, m1.y + n1.x};
         v[4] = C{m1.x + n1.y, m1.y - n1.x};

@@ -8,15 +8,20 @@
 //
 // A line (the n values one 1D transform works on) is a block floating-point
 // vector: integers v with the value v 2^-ke, ke one number per line, chosen
-// from the line's largest component and its 1-norm so that no partial sum of
-// the transform can overflow: every intermediate is a sum of inputs times
-// factors of modulus <= 1, so its modulus is at most the 1-norm and at most
-// the number of terms times the largest modulus (line_ke).  Twiddle products
-// come out divided by 4, which takes back most of the growth of the radix
-// before them, so the low bits stay in use through all stages: the rounding
-// noise stays below what FP64 sums leave (about 2^-53 of the line's 2-norm):
-// some 2^-61 of the 1-norm for inputs all alike, 2^-58 of it where a few
-// inputs dominate.
+// from the line's largest component and its 1-norm so that every partial sum
+// of the transform has a modulus below 2^62 (fx_ke, tile_ke): such a sum is one
+// of inputs times factors of modulus <= 1, so its modulus is at most the
+// 1-norm and at most the number of terms times the largest modulus.  The
+// butterflies form one value that is no such sum: x +- y of one complex value,
+// for fx_w32's 45-degree factors, up to sqrt 2 2^62.  So no value is doubled to
+// make room for a constant's 63 fraction bits (operator*, fx_w32), and every
+// product states what it can take.
+// A point charge reaches these bounds: one value carries its line's 1-norm.
+// Twiddle products come out divided by 4, which takes back most of the growth
+// of the radix before them, so the low bits stay in use through all stages:
+// the rounding noise stays below what FP64 sums leave (about 2^-53 of the
+// line's 2-norm): some 2^-61 of the 1-norm for inputs all alike, 2^-58 of it
+// where a few inputs dominate.
 //
 // Products: a is split into signed halves (ah 2^32 + al), w likewise, and
 //   a w / 2^64 = ah wh + (ah wl + al wh) / 2^32
@@ -57,27 +62,43 @@ __host__ __device__ constexpr int fx_lo(long long a) { return (int)(unsigned)(a 
 
 // a b + c
 __device__ __forceinline__ long long fx_mad(int a, int b, long long c) {
+#ifdef __CUDA_ARCH__
     long long d;
     asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
     return d;
+#else  // the arithmetic compiled for the host (tests)
+    return (long long)((unsigned long long)((long long)a * b) + (unsigned long long)c);
+#endif
 }
 __device__ __forceinline__ long long fx_high(long long a) { return (long long)(int)(a >> 32); }
 constexpr long long kFxHalf = 0x80000000LL;
 
-// a w / 2^64, w in signed halves
+// a w / 2^64, w in signed halves.  The cross terms are at most 2^31 (|ah| + |wh|),
+// which must stay below 2^63: |a| + |w| < 2^64.
 __device__ __forceinline__ long long fx_mul(long long a, int wh, int wl) {
     const int ah = fx_hi(a), al = fx_lo(a);
     return fx_mad(ah, wh, fx_high(fx_mad(ah, wl, fx_mad(al, wh, kFxHalf))));
 }
-// (x + i y) (wr + i wi) / 2^64, with u = -wi
+// (x + i y) (wr + i wi) / 2^64, with u = -wi.  The cross terms are below
+// 2^31 (|rh| + |ih|) + |x + i y| 2^-32 |rl + i il|, which must stay below 2^63:
+// with twiddles (|w| <= 2^62) 0.71 of it at the largest modulus, 2^62.
 __device__ __forceinline__ cfx fx_cmul(long long x, long long y, int rh, int rl, int ih, int il, int uh, int ul) {
     const int xh = fx_hi(x), xl = fx_lo(x), yh = fx_hi(y), yl = fx_lo(y);
     const long long p = fx_mad(xh, rl, fx_mad(xl, rh, fx_mad(yh, ul, fx_mad(yl, uh, kFxHalf))));
     const long long q = fx_mad(xh, il, fx_mad(xl, ih, fx_mad(yh, rl, fx_mad(yl, rh, kFxHalf))));
     return cfx{fx(fx_mad(xh, rh, fx_mad(yh, uh, fx_high(p))), 0), fx(fx_mad(xh, ih, fx_mad(yh, rh, fx_high(q))), 0)};
 }
-// constant c (63 fraction bits) times a, |a| < 2^62
-__device__ __forceinline__ fx operator*(fx c, fx a) { return fx(fx_mul(a.v << 1, fx_hi(c.v), fx_lo(c.v)), 0); }
+// Constants of modulus < 1, with 63 fraction bits: w 2 wraps to (w - k) 2^64, k
+// one of -1, 0, 1 (fx_whole), so that w a = k a + a (w - k) 2^64 / 2^64 and a need
+// not be doubled.
+__host__ __device__ constexpr long long fx_twice(long long c) { return (long long)((unsigned long long)c << 1); }
+__host__ __device__ constexpr int fx_whole(long long c) { return c >= 1LL << 62 ? 1 : c < -(1LL << 62) ? -1 : 0; }
+// constant c times a, |a| < 2^63
+__device__ __forceinline__ fx operator*(fx c, fx a) {
+    const long long w = fx_twice(c.v), r = fx_mul(a.v, fx_hi(w), fx_lo(w));
+    const int k = fx_whole(c.v);
+    return fx(k > 0 ? r + a.v : k < 0 ? r - a.v : r, 0);
+}
 
 // x w / 4 (D < 0) or x conj(w) / 4 (D > 0)
 template <int D> __device__ __forceinline__ cfx fx_twiddle(cfx x, fxw w) {
@@ -120,8 +141,15 @@ template <int D, int m> __device__ __forceinline__ cfx fx_w32(cfx a) {
         const fx t = sx > 0 ? (sy > 0 ? a.y + a.x : a.y - a.x) : (sy > 0 ? a.x - a.y : -(a.y + a.x));
         return cfx{c * u, c * t};
     } else {
-        constexpr long long c = fx_cos32(m), s = D * fx_cos32(m - 8);
-        return fx_cmul(a.x.v << 1, a.y.v << 1, fx_hi(c), fx_lo(c), fx_hi(s), fx_lo(s), fx_hi(-s), fx_lo(-s));
+        // cross terms at a modulus of 2^62: 0.93 2^63 for the worst of the constants
+        constexpr long long c = fx_cos32(m), s = D * fx_cos32(m - 8), wc = fx_twice(c), ws = fx_twice(s);
+        constexpr int kc = fx_whole(c), ks = fx_whole(s);
+        cfx r = fx_cmul(a.x.v, a.y.v, fx_hi(wc), fx_lo(wc), fx_hi(ws), fx_lo(ws), fx_hi(-ws), fx_lo(-ws));
+        if constexpr (kc > 0) r = cfx{r.x + a.x, r.y + a.y};
+        if constexpr (kc < 0) r = cfx{r.x - a.x, r.y - a.y};
+        if constexpr (ks > 0) r = cfx{r.x - a.y, r.y + a.x};
+        if constexpr (ks < 0) r = cfx{r.x + a.y, r.y - a.x};
+        return r;
     }
 }
 

@@ -35,6 +35,34 @@ __device__ __forceinline__ int fx_em(int hmax) { return max(hmax >> 20, 1) - 102
 // the range of em in which fx_fabs, fx_of and fx_of_p hold
 __device__ __forceinline__ bool fx_far(int em) { return em < -60 || em > 90; }
 
+// ---- the scale of a line with a runtime schedule (kernels_impl.cuh)
+// s <= 2^em * (some 2^12) in units of 2^(em - 16), rounded up; |em| < 100
+__device__ __forceinline__ unsigned tile_units(float s, int em) {
+    return (unsigned)(s * __int_as_float((127 + 16 - em) << 23)) + 1u;
+}
+// fx_ke of a runtime schedule (5s, 3s, 8s, last): modulus <= 2^B after every
+// stage, each stage after the first dividing by 4 beforehand
+__device__ __forceinline__ int tile_ke(const Stages &st, int em, int eL, int B) {
+    int eb = -100000, g = 0, d = 0;
+    auto stage = [&](int grow) {
+        g += grow;
+        eb = max(eb, min(em + 1 + g, eL) - d);
+        d += 2;
+    };
+    for (int i = 0; i < st.n5; ++i) stage(3);
+    for (int i = 0; i < st.n3; ++i) stage(2);
+    for (int i = 0; i < st.n8; ++i) stage(3);
+    if (st.last) stage(st.last == 4 ? 2 : 1);
+    return B - max(eb, min(em + 1, eL));  // (a transform of length 1 has no stage)
+}
+__device__ __forceinline__ int tile_log2(const Stages &st) {
+    return 3 * st.n5 + 2 * st.n3 + 3 * st.n8 + (st.last == 4 ? 2 : st.last == 2 ? 1 : 0) + 1;
+}
+// twice the number of stages that divide by 4
+__device__ __forceinline__ int tile_div(const Stages &st) {
+    return 2 * max(st.n5 + st.n3 + st.n8 + (st.last ? 1 : 0) - 1, 0);
+}
+
 // PX, PY: that component through the FP64 pipe.  A pass mixes the two ways so
 // that neither pipe waits for the other.
 template <bool PX, bool PY> __device__ __forceinline__ cfx fx_conv(const cfx &v, const FxScale &sc) {
