@@ -9,6 +9,7 @@
 // (96) 3.45, with six 3.92; the generic engine's kernel takes 9.07.  A work
 // item is a run of tiles of one pass of about 8K points: the cursor, the item's
 // descriptor and the wait are paid for once per item.
+#include <algorithm>
 #include <cuda/atomic>
 
 #include "../../include/fsp.h"
@@ -198,10 +199,14 @@ size_t fast_batch_smem(int N) {
     }
     return 0;
 }
-// Sets the shared-memory attribute too, so that the launch can be captured.
+// Sets the shared-memory attribute too, so that the launch can be captured: to
+// what the largest size needs whatever this batch holds, because it is one
+// value for the process and other live batches are captured again under it.
 int fast_batch_blocks_per_sm(size_t smem) {
     int nb = 0;
-    cudaFuncSetAttribute(fast::k_batch_fast, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    size_t most = 0;
+    for (int N : {32, 48, 64, 96, 128, 160, 192, 256}) most = std::max(most, fast_batch_smem(N));
+    cudaFuncSetAttribute(fast::k_batch_fast, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fast::k_batch_fast, fast::kThreads, smem) != cudaSuccess)
         return 0;
     return nb;

@@ -1,0 +1,95 @@
+"""The library's host side on a fake CUDA runtime (tests/host/fake_cudart.cpp):
+calls that fail, several devices, little memory.  Nothing here needs a GPU."""
+import ctypes
+import glob
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2405_02603_gb300 import build as B
+
+OK = 0
+F64, F32, F64_DF = 0, 1, 2
+HE = 0
+VP = ctypes.c_void_p
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    here = os.path.dirname(os.path.abspath(__file__))
+    objects = lambda: glob.glob(os.path.join(B.OUT_DIR, "*.o"))  # noqa: E731
+    B.build(force=len(objects()) < len(B.sources()))
+    names = {os.path.basename(s)[:-3] + ".o" for s in B.sources()}
+    out = str(tmp_path_factory.mktemp("fake") / "libfsp_fake.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc()))), "include")
+    # its own CUDA runtime, whatever else the process has loaded
+    subprocess.run(["g++", "-std=c++17", "-O1", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I", cuda,
+                    os.path.join(here, "host", "fake_cudart.cpp")] +
+                   [o for o in objects() if os.path.basename(o) in names] + ["-o", out], check=True)
+    L = ctypes.CDLL(out)
+    i, d = ctypes.c_int, ctypes.c_double
+    L.fsp_plan_create.argtypes = [ctypes.POINTER(VP), i, d, d, i, i, VP]
+    L.fsp_solve.argtypes = [VP, VP, VP, VP]
+    L.fsp_plan_destroy.argtypes = [VP]
+    L.fsp_batch_create.argtypes = [ctypes.POINTER(VP), ctypes.POINTER(VP), ctypes.POINTER(VP), ctypes.POINTER(VP), i, VP]
+    for f in ("launch", "wait", "autotune"):
+        getattr(L, "fsp_batch_" + f).argtypes = [VP, VP]
+    L.fsp_batch_set_timeout.argtypes = [VP, d]
+    L.fsp_batch_set_form.argtypes = [VP, i]
+    L.fsp_batch_destroy.argtypes = [VP]
+    for f in ("fake_used", "fake_idle"):
+        getattr(L, f).restype = ctypes.c_size_t
+    L.fake_violations.restype = ctypes.c_long
+    L.fake_capacity.argtypes = [ctypes.c_size_t]
+    L.fake_fail.argtypes = [ctypes.c_char_p, i, i]
+    L.fake_failed.argtypes = [ctypes.c_char_p]
+    return L
+
+
+def plan(L, N, dtype=F64, algo=HE):
+    p = VP()
+    assert L.fsp_plan_create(ctypes.byref(p), N, 1.0, 1.0 / N, algo, dtype, None) == OK
+    return p
+
+
+class Arrays:
+    """16-byte aligned arrays of N^3 reals."""
+
+    def __init__(self, Ns, dtype):
+        self.keep = [np.zeros(n ** 3 + 4, np.float32 if dtype == F32 else np.float64) for n in Ns]
+        self.ptrs = (VP * len(Ns))(*[(a.ctypes.data + 15) // 16 * 16 for a in self.keep])
+
+
+class BatchOf:
+    def __init__(self, L, Ns, dtype):
+        self.L, self.plans = L, [plan(L, N, dtype) for N in Ns]
+        self.rho, self.phi = Arrays(Ns, dtype), Arrays(Ns, dtype)
+        self.b = VP()
+        assert L.fsp_batch_create(ctypes.byref(self.b), (VP * len(Ns))(*[p.value for p in self.plans]), self.rho.ptrs,
+                                  self.phi.ptrs, len(Ns), None) == OK
+
+    def usable(self):
+        """Launches, on live memory."""
+        before = self.L.fake_violations()
+        return self.L.fsp_batch_launch(self.b, None) == OK and self.L.fsp_batch_wait(self.b, None) == OK and \
+            self.L.fake_violations() == before
+
+    def close(self):
+        assert self.L.fsp_batch_destroy(self.b) == OK
+        for p in self.plans:
+            assert self.L.fsp_plan_destroy(p) == OK
+
+
+def test_batches_of_different_sizes_live_together(fake):
+    """The kernel's shared-memory attribute belongs to the process: a batch of
+    small plans must not take it from one of large plans."""
+    L = fake
+    L.fake_reset(1)
+    big = BatchOf(L, [160, 128], F32)
+    small = BatchOf(L, [32, 32], F32)
+    assert L.fsp_batch_set_timeout(big.b, 500.0) == OK
+    assert big.usable() and small.usable()
+    big.close()
+    small.close()
