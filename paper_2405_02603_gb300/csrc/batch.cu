@@ -132,7 +132,7 @@ template <typename T> cudaError_t launch_batch_kernel(const BatchLaunch &L, cuda
 
 template <typename T> int batch_blocks_per_sm(int threads, size_t smem) {
     int nb = 0;
-    cudaFuncSetAttribute(k_batch<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_batch<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxTileSmem);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch<T>, threads, smem) != cudaSuccess) return 0;
     return nb;
 }

@@ -10,6 +10,7 @@
 #include "fast.cuh"
 #include "fx_line.cuh"
 #include "kernels.cuh"
+#include "tiles.h"
 
 namespace fsp {
 
@@ -550,14 +551,14 @@ template <typename T> size_t rows_smem_bytes(const RowsArgs &a) {
     return (size_t)(a.N + 1) * smem_pitch(a.lgL) * sizeof(cx_t<T>);
 }
 
-template <typename K> static cudaError_t set_smem(K kernel, size_t bytes) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+template <typename K> static cudaError_t set_smem(K kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxTileSmem);
 }
 
 template <typename T, int IN, int OUT, int MODE> cudaError_t launch_lines(const LinesArgs &a, cudaStream_t s) {
     const size_t sm = lines_smem_bytes<T>(a);
     auto kern = k_lines<T, IN, OUT, MODE>;
-    cudaError_t e = set_smem(kern, sm);
+    cudaError_t e = set_smem(kern);
     if (e != cudaSuccess) return e;
     const int nl = lines_pair(IN) ? (a.nlines + 1) / 2 : a.nlines;
     dim3 grid((unsigned)((nl + (1 << a.lgL) - 1) >> a.lgL), (unsigned)a.nbatch);
@@ -566,7 +567,7 @@ template <typename T, int IN, int OUT, int MODE> cudaError_t launch_lines(const 
 
 template <typename T> cudaError_t launch_r2c_rows(const RowsArgs &a, cudaStream_t s) {
     const size_t sm = rows_smem_bytes<T>(a);
-    cudaError_t e = set_smem(k_r2c_rows<T>, sm);
+    cudaError_t e = set_smem(k_r2c_rows<T>);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)((a.nrows + (1 << a.lgL) - 1) >> a.lgL));
     return launch_pass(k_r2c_rows<T>, grid, (1 << a.lgL) * a.tpl, sm, s, a);
@@ -574,7 +575,7 @@ template <typename T> cudaError_t launch_r2c_rows(const RowsArgs &a, cudaStream_
 
 template <typename T> cudaError_t launch_c2r_rows(const RowsArgs &a, cudaStream_t s) {
     const size_t sm = rows_smem_bytes<T>(a);
-    cudaError_t e = set_smem(k_c2r_rows<T>, sm);
+    cudaError_t e = set_smem(k_c2r_rows<T>);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)((a.nrows + (1 << a.lgL) - 1) >> a.lgL));
     return launch_pass(k_c2r_rows<T>, grid, (1 << a.lgL) * a.tpl, sm, s, a);

@@ -46,13 +46,19 @@ inline int threads_per_line(const Stages &st) {
     }
 }
 
-// Lines per CTA (2^lgL): as many as wanted, within 512 threads and 200 KB of
-// shared memory (positions x (L+1) complex elements).
+// Dynamic shared memory of a tile, at most.  A kernel's limit on it belongs to
+// the process, not to a launch, so every launch sets it to this value: with
+// its own need, a launch could take the limit from one that another thread
+// is about to make, or from a batch that is captured again later.
+constexpr size_t kMaxTileSmem = 200 * 1024;
+
+// Lines per CTA (2^lgL): as many as wanted, within 512 threads and
+// kMaxTileSmem of shared memory (positions x (L+1) complex elements).
 inline bool choose_tile(int positions, int tpl, size_t csize, int want_lgL, int &lgL) {
     for (lgL = want_lgL; lgL >= 0; --lgL) {
         const int L = 1 << lgL;
         const size_t sm = (size_t)positions * (L + 1) * csize;
-        if (L * tpl <= 512 && sm <= 200 * 1024) return true;
+        if (L * tpl <= 512 && sm <= kMaxTileSmem) return true;
     }
     return false;
 }

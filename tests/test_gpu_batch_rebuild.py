@@ -7,7 +7,7 @@ from conftest import to_dev
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dtype,Ns", [("f32", [[256, 160], [32], [96, 48]])])
+@pytest.mark.parametrize("dtype,Ns", [("f32", [[256, 160], [32], [96, 48]]), ("f64", [[75, 128], [16], [50]])])
 def test_live_batches_of_different_sizes(fsp, dtype, Ns):
     import torch
     batches = []

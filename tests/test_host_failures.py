@@ -82,13 +82,14 @@ class BatchOf:
             assert self.L.fsp_plan_destroy(p) == OK
 
 
-def test_batches_of_different_sizes_live_together(fake):
+@pytest.mark.parametrize("dtype,Ns", [(F32, [160, 128]), (F64, [75, 128])])
+def test_batches_of_different_sizes_live_together(fake, dtype, Ns):
     """The kernel's shared-memory attribute belongs to the process: a batch of
     small plans must not take it from one of large plans."""
     L = fake
     L.fake_reset(1)
-    big = BatchOf(L, [160, 128], F32)
-    small = BatchOf(L, [32, 32], F32)
+    big = BatchOf(L, Ns, dtype)
+    small = BatchOf(L, [32, 32], dtype)
     assert L.fsp_batch_set_timeout(big.b, 500.0) == OK
     assert big.usable() and small.usable()
     big.close()
