@@ -1690,14 +1690,8 @@ fsp_status fsp_fft_c2c(int n, int count, fsp_dtype dtype, int sign, const void *
 }  // extern "C"
 
 // ------------------------------------------------------------- batches --
-struct fsp_batch {
-    uint64_t magic = 0;
-    int device = 0, count = 0;
-    fsp_dtype dtype = FSP_F64;
-    std::vector<fsp_plan *> plans;
-    std::vector<const void *> rho;
-    std::vector<void *> phi;
-    std::map<int, std::pair<int, int>> shape;  // per N: (lgL_row, lgL_col) of its tiles
+// What batch_build makes of a batch: work list, device arrays and graph.
+struct BatchBuild {
     std::vector<BatchSolve> solves;
     std::vector<BatchSeg> segs;
     int total = 0;
@@ -1708,14 +1702,26 @@ struct fsp_batch {
     BatchLaunch launch{};
     // every plan on the specialised FP32 kernels: their own persistent kernel
     bool fast = false;
-    bool tuning = false;  // the autotuner at work: it times the generic engine's shapes
     FastBatchSolve *d_fsolves = nullptr;
     FastBatchItem *d_items = nullptr;
     FastBatchLaunch flaunch{};
-    double timeout_ms = 1000.0;
-    int form = 0;  // 0: one persistent kernel; 1: the solves' own launches on several streams
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+};
+// ... and what it makes it of.
+struct BatchConfig {
+    int device = 0, count = 0;
+    fsp_dtype dtype = FSP_F64;
+    std::vector<fsp_plan *> plans;
+    std::vector<const void *> rho;
+    std::vector<void *> phi;
+    std::map<int, std::pair<int, int>> shape;  // per N: (lgL_row, lgL_col) of its tiles
+    bool tuning = false;  // the autotuner at work: it times the generic engine's shapes
+    double timeout_ms = 1000.0;
+    int form = 0;  // 0: one persistent kernel; 1: the solves' own launches on several streams
+};
+struct fsp_batch : BatchConfig, BatchBuild {
+    uint64_t magic = 0;
 };
 
 namespace {
@@ -1728,16 +1734,16 @@ bool batch_live(const fsp_batch *b) {
     return b && g_batches.count(b) && b->magic == kBatchMagic;
 }
 
-void batch_free_lists(fsp_batch *b) {
-    for (void *q : {(void *)b->d_solves, (void *)b->d_segs, (void *)b->d_ctl, (void *)b->d_fsolves, (void *)b->d_items})
+void batch_release(BatchBuild &b) {
+    if (b.exec) cudaGraphExecDestroy(b.exec);
+    if (b.graph) cudaGraphDestroy(b.graph);
+    for (void *q : {(void *)b.d_solves, (void *)b.d_segs, (void *)b.d_ctl, (void *)b.d_fsolves, (void *)b.d_items})
         if (q) dev_free(q);
-    b->d_solves = nullptr, b->d_segs = nullptr, b->d_ctl = nullptr, b->d_fsolves = nullptr, b->d_items = nullptr;
+    b = BatchBuild();
 }
 
 void batch_free(fsp_batch *b) {
-    if (b->exec) cudaGraphExecDestroy(b->exec);
-    if (b->graph) cudaGraphDestroy(b->graph);
-    batch_free_lists(b);
+    batch_release(*b);
     b->magic = 0;
     delete b;
 }
@@ -1799,12 +1805,18 @@ FastBatchSolve fast_batch_solve_of(const fsp_plan *p, const void *rho, void *phi
     return b;
 }
 
+// (Re)capture a batch's graph; on failure the one it had stays.
 fsp_status batch_build_graph(fsp_batch *b) {
-    if (b->exec) cudaGraphExecDestroy(b->exec), b->exec = nullptr;
-    if (b->graph) cudaGraphDestroy(b->graph), b->graph = nullptr;
-    b->launch.timeout_ns = b->flaunch.timeout_ns = (unsigned long long)(b->timeout_ms * 1e6);
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    BatchLaunch launch = b->launch;
+    FastBatchLaunch flaunch = b->flaunch;
+    launch.timeout_ns = flaunch.timeout_ns = (unsigned long long)(b->timeout_ms * 1e6);
     cudaStream_t cs;
-    if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return FSP_ECUDA;
+    if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
+        cudaGetLastError();
+        return FSP_ECUDA;
+    }
     // form 1: kStreams capture streams forked from cs; a plan's solves stay on
     // one stream (they share its workspace), plans are dealt round-robin
     constexpr int kStreams = 8;
@@ -1822,9 +1834,9 @@ fsp_status batch_build_graph(fsp_batch *b) {
         cudaError_t e1 = cudaMemsetAsync(b->d_ctl, 0, b->ctl_bytes, cs);
         cudaError_t e2 = e1;
         if (e1 == cudaSuccess && b->form == 0) {
-            e2 = b->fast               ? launch_fast_batch(b->flaunch, cs)
-                 : b->dtype == FSP_F64 ? launch_batch_kernel<double>(b->launch, cs)
-                                       : launch_batch_kernel<float>(b->launch, cs);
+            e2 = b->fast               ? launch_fast_batch(flaunch, cs)
+                 : b->dtype == FSP_F64 ? launch_batch_kernel<double>(launch, cs)
+                                       : launch_batch_kernel<float>(launch, cs);
         } else if (e1 == cudaSuccess) {
             e2 = cudaEventRecord(fev[kStreams], cs);
             for (int i = 0; i < kStreams && e2 == cudaSuccess; ++i) e2 = cudaStreamWaitEvent(fs[i], fev[kStreams], 0);
@@ -1840,7 +1852,7 @@ fsp_status batch_build_graph(fsp_batch *b) {
                 if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(cs, fev[i], 0);
             }
         }
-        e = cudaStreamEndCapture(cs, &b->graph);
+        e = cudaStreamEndCapture(cs, &graph);
         if (e == cudaSuccess) e = e2;
     }
     for (int i = 0; i < kStreams; ++i) {
@@ -1848,9 +1860,17 @@ fsp_status batch_build_graph(fsp_batch *b) {
         if (fev[i]) cudaEventDestroy(fev[i]);
     }
     if (fev[kStreams]) cudaEventDestroy(fev[kStreams]);
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&b->exec, b->graph, 0);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
     cudaStreamDestroy(cs);
-    return cuda_status(e);
+    if (e != cudaSuccess) {
+        if (graph) cudaGraphDestroy(graph);
+        cudaGetLastError();  // it must not be taken for a later launch's
+        return FSP_ECUDA;
+    }
+    if (b->exec) cudaGraphExecDestroy(b->exec);
+    if (b->graph) cudaGraphDestroy(b->graph);
+    b->graph = graph, b->exec = exec, b->launch = launch, b->flaunch = flaunch;
+    return FSP_OK;
 }
 
 }  // namespace
@@ -1869,7 +1889,7 @@ void batch_tiles(const fsp_batch *b, const fsp_plan *p, TileCfg &row, TileCfg &c
     if (choose_tile(2 * p->N, c.tpl, csize, it->second.second, c.lgL)) col = c;
 }
 
-// batch_build for plans that are all on the specialised FP32 kernels.
+// batch_build_new for plans that are all on the specialised FP32 kernels.
 fsp_status batch_build_fast(fsp_batch *b, cudaStream_t s) {
     const int count = b->count;
     std::vector<FastBatchSolve> solves;
@@ -1882,7 +1902,6 @@ fsp_status batch_build_fast(fsp_batch *b, cudaStream_t s) {
         smem = std::max(smem, fast_batch_smem(b->plans[i]->N));
     }
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->plans[x]->N > b->plans[y]->N; });
-    b->segs.clear();
     for (int pass = 0; pass < 5; ++pass)
         for (int i : order) {
             int ntiles[5], group[5];
@@ -1919,17 +1938,14 @@ fsp_status batch_build_fast(fsp_batch *b, cudaStream_t s) {
     return batch_build_graph(b);
 }
 
-// (Re)build descriptors, work list, device arrays and graph of a batch.
-fsp_status batch_build(fsp_batch *b, cudaStream_t s) {
+// Descriptors, work list, device arrays and graph of a batch that has none.
+fsp_status batch_build_new(fsp_batch *b, cudaStream_t s) {
     const int count = b->count;
-    batch_free_lists(b);
     b->fast = b->dtype == FSP_F32_MIXED && !b->tuning &&
               std::all_of(b->plans.begin(), b->plans.end(),
                           [](const fsp_plan *p) { return p->fast && p->W1 && fast_batch_has(p->N); });
     if (b->fast) return batch_build_fast(b, s);
     const size_t csize = 2 * b->plans[0]->rsize;
-    b->solves.clear();
-    b->segs.clear();
     int threads = 32;
     size_t smem = 0;
     for (int i = 0; i < count; ++i) {
@@ -1976,6 +1992,21 @@ fsp_status batch_build(fsp_batch *b, cudaStream_t s) {
     b->launch.grid = (unsigned)std::min<long long>((long long)sms * per_sm, b->total);
     b->launch.threads = threads, b->launch.smem = smem;
     return batch_build_graph(b);
+}
+
+// Build a batch, or build it again: the new build takes the old one's place
+// when it is complete, and a failed one leaves the batch as it was (its graph
+// must never outlive the arrays it uses).
+fsp_status batch_build(fsp_batch *b, cudaStream_t s) {
+    fsp_batch n;
+    static_cast<BatchConfig &>(n) = *b;
+    const fsp_status st = batch_build_new(&n, s);
+    if (st == FSP_OK)
+        std::swap(static_cast<BatchBuild &>(*b), static_cast<BatchBuild &>(n));
+    else
+        cudaGetLastError();
+    batch_release(n);
+    return st;
 }
 
 }  // namespace
@@ -2030,8 +2061,11 @@ extern "C" fsp_status fsp_batch_wait(fsp_batch *b, fsp_stream stream) {
 
 extern "C" fsp_status fsp_batch_set_timeout(fsp_batch *b, double ms) {
     if (!batch_live(b) || !(ms > 0.0) || ms > 3.6e6) return FSP_EINVAL;
+    const double before = b->timeout_ms;
     b->timeout_ms = ms;
-    return batch_build_graph(b);
+    const fsp_status st = batch_build_graph(b);
+    if (st != FSP_OK) b->timeout_ms = before;
+    return st;
 }
 
 extern "C" fsp_status fsp_batch_set_form(fsp_batch *b, int form) {
@@ -2039,8 +2073,11 @@ extern "C" fsp_status fsp_batch_set_form(fsp_batch *b, int form) {
     if (form == 1)
         for (const fsp_plan *p : b->plans)
             if (!p->W1) return FSP_EINVAL;
+    const int before = b->form;
     b->form = form;
-    return batch_build_graph(b);
+    const fsp_status st = batch_build_graph(b);
+    if (st != FSP_OK) b->form = before;
+    return st;
 }
 
 extern "C" fsp_status fsp_batch_inject_stall(fsp_batch *b) {
@@ -2102,7 +2139,10 @@ fsp_status batch_tune(fsp_batch *b, cudaStream_t s) {
                 (which ? trial.second : trial.first) = lg;
                 if (trial == keep) continue;
                 b->shape[N] = trial;
-                if ((st = batch_build(b, s)) != FSP_OK) return st;
+                if ((st = batch_build(b, s)) != FSP_OK) {
+                    b->shape[N] = keep;
+                    return st;
+                }
                 const double t = time_batch(b, s, 3);
                 if (t > 0 && t < best)
                     best = t;

@@ -94,3 +94,34 @@ def test_batches_of_different_sizes_live_together(fake, dtype, Ns):
     assert big.usable() and small.usable()
     big.close()
     small.close()
+
+
+@pytest.mark.parametrize("dtype", [F64, F32])
+@pytest.mark.parametrize("call", [b"alloc", b"copy", b"stream", b"capture", b"instantiate"])
+def test_failed_rebuild_leaves_the_batch(fake, dtype, call):
+    """Whichever of its calls fails, the autotuner returns an error and the
+    batch runs on, with live memory; so do set_timeout and set_form."""
+    L = fake
+    L.fake_reset(1)
+    b = BatchOf(L, [32, 64] if dtype == F32 else [16, 20], dtype)
+    assert b.usable()
+    nth, failed = 0, 0
+    while True:
+        L.fake_fail(call, nth, 3 if call == b"alloc" else 1)  # an allocation is tried three times
+        st = L.fsp_batch_autotune(b.b, None)
+        hit = L.fake_failed(call)
+        L.fake_fail_none()
+        assert b.usable(), nth
+        if not hit:
+            break
+        failed += st != OK
+        nth += 1 if nth < 12 else 7
+    assert failed >= 3 and st == OK
+    if call in (b"stream", b"capture", b"instantiate"):
+        for change in (lambda: L.fsp_batch_set_timeout(b.b, 20.0), lambda: L.fsp_batch_set_form(b.b, 1)):
+            L.fake_fail(call, 0, 1)
+            assert change() != OK
+            L.fake_fail_none()
+            assert b.usable()
+            assert change() == OK and b.usable()
+    b.close()
