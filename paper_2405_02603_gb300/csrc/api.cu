@@ -160,6 +160,7 @@ constexpr unsigned long long kPoolKeep = 1ull << 30;
 struct DevPool {
     cudaMemPool_t pool = nullptr;
     cudaStream_t stream = nullptr;
+    int dev = 0;
 };
 std::mutex g_pool_mu;
 std::map<int, DevPool> g_pools;
@@ -184,6 +185,7 @@ DevPool dev_pool() {
     auto it = g_pools.find(dev);
     if (it != g_pools.end()) return it->second;
     DevPool d;
+    d.dev = dev;
     cudaMemPoolProps props{};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
@@ -228,9 +230,27 @@ cudaError_t plain_malloc(void **p, size_t bytes) {
     return e;
 }
 
-// As cudaFree: everything enqueued on the device before is complete.  Where
-// waiting is refused (a stream in capture) the buffer is kept until a later
-// free can wait: another plan must not get memory that is still in use.
+// Makes a device current for a scope (a plan may be destroyed while another
+// device is).
+struct DeviceScope {
+    int prev = -1;
+    bool ok;
+    explicit DeviceScope(int dev) {
+        ok = cudaGetDevice(&prev) == cudaSuccess;
+        if (ok && prev != dev)
+            ok = cudaSetDevice(dev) == cudaSuccess;
+        else
+            prev = -1;  // nothing to put back
+    }
+    ~DeviceScope() {
+        if (prev >= 0) cudaSetDevice(prev);
+    }
+};
+
+// As cudaFree: everything enqueued before on the buffer's own device is
+// complete.  Where waiting is refused (a stream in capture) the buffer is kept
+// until a later free can wait for that device: another plan must not get
+// memory that is still in use.
 void plain_free(void *p) {
     DevPool d;
     {
@@ -249,12 +269,19 @@ void plain_free(void *p) {
         cudaFreeAsync(p, d.stream);
         return;
     }
-    const bool idle = !t_free_stream && cudaDeviceSynchronize() == cudaSuccess;
+    DeviceScope scope(d.dev);
+    const bool idle = !t_free_stream && scope.ok && cudaDeviceSynchronize() == cudaSuccess;
     std::lock_guard<std::mutex> lk(g_pool_mu);
     g_unsynced.emplace_back(p, d);
     if (!idle) return;
-    for (const auto &q : g_unsynced) cudaFreeAsync(q.first, q.second.stream);
-    g_unsynced.clear();
+    std::vector<std::pair<void *, DevPool>> others;
+    for (const auto &q : g_unsynced) {
+        if (q.second.dev == d.dev)
+            cudaFreeAsync(q.first, q.second.stream);
+        else
+            others.push_back(q);
+    }
+    g_unsynced.swap(others);
 }
 
 void dev_free(void *p) {

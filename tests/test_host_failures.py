@@ -125,3 +125,35 @@ def test_failed_rebuild_leaves_the_batch(fake, dtype, call):
             assert b.usable()
             assert change() == OK and b.usable()
     b.close()
+
+
+def test_buffers_wait_for_their_own_device(fake):
+    """A buffer goes back to the pool when the work on its own device is done,
+    whichever device is current, also when a capture kept it from going at first."""
+    L = fake
+    L.fake_reset(2)
+    used = [L.fake_used(d) for d in (0, 1)]
+    a = Arrays([16, 16], F64)
+    on = {}
+    for d in (0, 1):
+        assert L.cudaSetDevice(d) == 0
+        on[d] = [plan(L, 16), plan(L, 16)]
+    assert L.fsp_solve(on[1][0], a.ptrs[0], a.ptrs[1], None) == OK  # device 1 is current
+    L.cudaSetDevice(0)
+    assert L.fsp_plan_destroy(on[1][0]) == OK
+    assert L.fake_violations() == 0
+    # device 0: refused while a stream is in capture, then freed from device 1
+    stream, graph = VP(), VP()
+    assert L.cudaStreamCreateWithFlags(ctypes.byref(stream), 1) == 0
+    assert L.fsp_solve(on[0][0], a.ptrs[0], a.ptrs[1], None) == OK
+    L.cudaStreamBeginCapture(stream, 1)
+    L.fsp_plan_destroy(on[0][0])
+    L.cudaStreamEndCapture(stream, ctypes.byref(graph))
+    L.cudaSetDevice(1)
+    assert L.fsp_plan_destroy(on[1][1]) == OK
+    assert L.fake_violations() == 0
+    assert L.fake_used(0) > used[0]
+    L.cudaSetDevice(0)
+    assert L.fsp_plan_destroy(on[0][1]) == OK
+    assert L.fake_violations() == 0
+    assert [L.fake_used(d) for d in (0, 1)] == used
