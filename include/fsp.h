@@ -228,8 +228,17 @@ fsp_status fsp_plan_inject_stall(fsp_plan *plan);
 
 /* Release the plan and all its device memory.  Waits for the device first.
  * A destroyed or unknown pointer returns FSP_EINVAL (plans are tracked in a
- * registry, so a stale pointer is detected instead of dereferenced). */
+ * registry, so a stale pointer is detected instead of dereferenced).
+ *
+ * Of the memory of destroyed plans and of plan-time temporaries the library
+ * keeps up to 1 GiB per device for the next plan (buffers of up to 256 MiB).
+ * Its own allocations take that memory back when the device is full; other
+ * allocators of the process cannot reach it until fsp_memory_trim. */
 fsp_status fsp_plan_destroy(fsp_plan *plan);
+
+/* Give the unused device memory that the library keeps back to the driver, on
+ * every device.  Live plans are not touched. */
+fsp_status fsp_memory_trim(void);
 
 /*
  * fsp_plan_set_timing -- per-pass timing hook.  With nevents == 6, every later

@@ -545,6 +545,12 @@ def solve_noalloc(S, rho, phi, stream=None):
     return phi
 
 
+def memory_trim():
+    """Give device memory that the library keeps for the next plan (at most
+    1 GiB per device) back to the driver, for other allocators."""
+    check(lib().fsp_memory_trim(), "fsp_memory_trim")
+
+
 def fft_c2c(x, sign=-1, stream=None):
     """Batched 1D FFTs along the last axis of a complex CUDA tensor (library kernels)."""
     import torch
@@ -560,7 +566,7 @@ def fft_c2c(x, sign=-1, stream=None):
     return out
 
 
-__all__ = ["autotune", "tuning_get", "tuning_set", "Plan", "Batch", "Server", "solve_batched", "FspError", "kernel_T", "fft_c2c", "solve_noalloc", "lib", "check", "library_path", "ALGOS", "DTYPES"]
+__all__ = ["autotune", "tuning_get", "tuning_set", "Plan", "Batch", "Server", "solve_batched", "FspError", "kernel_T", "fft_c2c", "solve_noalloc", "memory_trim", "lib", "check", "library_path", "ALGOS", "DTYPES"]
 
 
 def device_host_numa(device=None):

@@ -33,6 +33,7 @@
 #include "internal.h"
 
 using namespace fsp;
+using fsp::internal::device_malloc;
 
 namespace {
 
@@ -98,7 +99,7 @@ __global__ void k_abs_max(const double *x, long long n, unsigned long long *out)
 
 fsp_status abs_max(const double *x, long long n, cudaStream_t s, double *out) {
     unsigned long long *d = nullptr, h = 0;
-    if (cudaMalloc(&d, sizeof(*d)) != cudaSuccess) {
+    if (device_malloc((void **)&d, sizeof(*d)) != cudaSuccess) {
         cudaGetLastError();
         return FSP_ENOMEM;
     }
@@ -137,7 +138,7 @@ __global__ void k_count_not(const unsigned char *a, size_t n, unsigned char v, u
 // changed guard bytes around the guarded buffer at p (synchronous)
 unsigned long long guard_bad(const void *p, const Guarded &g) {
     unsigned long long *d = nullptr, h = 0;
-    if (cudaMalloc(&d, sizeof(*d)) != cudaSuccess) return ~0ull;
+    if (device_malloc((void **)&d, sizeof(*d)) != cudaSuccess) return ~0ull;
     cudaMemset(d, 0, sizeof(*d));
     const unsigned char *base = static_cast<const unsigned char *>(g.base);
     k_count_not<<<64, 256>>>(base, kGuard, kGuardByte, d);
@@ -153,8 +154,10 @@ unsigned long long guard_bad(const void *p, const Guarded &g) {
 // domains) allocates about ten buffers and frees them, and cudaMalloc and
 // cudaFree took most of its time (a VG-DCT plan and one solve at N = 96: 1.3 of
 // 2.3 ms).  The pool keeps at most kPoolKeep unused bytes (the driver returns
-// the rest at the next synchronisation), buffers above kPoolMax bypass it, and
-// an allocation that fails elsewhere empties it and tries again.
+// the rest at the next synchronisation) and buffers above kPoolMax bypass it.
+// Every other allocation of the library goes through device_malloc, which
+// empties the pool and tries again when the device is full; for allocators
+// outside the library there is fsp_memory_trim.
 constexpr size_t kPoolMax = (size_t)256 << 20;
 constexpr unsigned long long kPoolKeep = 1ull << 30;
 struct DevPool {
@@ -203,6 +206,12 @@ DevPool dev_pool() {
     return d;
 }
 
+// gives the pool's unused memory back to the driver
+cudaError_t pool_trim(const DevPool &d) {
+    const cudaError_t e = cudaStreamSynchronize(d.stream);  // frees enqueued there
+    return e != cudaSuccess ? e : cudaMemPoolTrimTo(d.pool, 0);
+}
+
 cudaError_t plain_malloc(void **p, size_t bytes) {
     const DevPool d = dev_pool();
     if (d.pool && bytes <= kPoolMax) {
@@ -220,14 +229,7 @@ cudaError_t plain_malloc(void **p, size_t bytes) {
         }
         cudaGetLastError();
     }
-    cudaError_t e = cudaMalloc(p, bytes);
-    if (e == cudaErrorMemoryAllocation && d.pool) {
-        cudaGetLastError();
-        cudaStreamSynchronize(d.stream);
-        cudaMemPoolTrimTo(d.pool, 0);
-        e = cudaMalloc(p, bytes);
-    }
-    return e;
+    return device_malloc(p, bytes);
 }
 
 // Makes a device current for a scope (a plan may be destroyed while another
@@ -307,7 +309,7 @@ void dev_free(void *p) {
 cudaError_t dev_malloc(void **p, size_t bytes) {
     if (!t_guard) return plain_malloc(p, bytes);
     void *base = nullptr;
-    cudaError_t e = cudaMalloc(&base, bytes + 2 * kGuard);
+    cudaError_t e = device_malloc(&base, bytes + 2 * kGuard);
     if (e != cudaSuccess) return e;
     if ((e = cudaMemset(base, kGuardByte, bytes + 2 * kGuard)) != cudaSuccess) {
         cudaFree(base);
@@ -1209,6 +1211,16 @@ fsp_status plan_create_impl(fsp_plan **out, int N, double L, double h, fsp_algo 
 namespace fsp {
 namespace internal {
 
+cudaError_t device_malloc(void **p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    const DevPool d = dev_pool();
+    if (!d.pool) return e;
+    cudaGetLastError();
+    pool_trim(d);
+    return cudaMalloc(p, bytes);
+}
+
 fsp_status spectrum_plan_create(fsp_plan **out, int N, double L, fsp_algo algo, fsp_dtype dtype, cudaStream_t s) {
     return plan_create_impl(out, N, L, L / N, algo, dtype, reinterpret_cast<fsp_stream>(s), false);
 }
@@ -1564,6 +1576,24 @@ fsp_status fsp_plan_destroy(fsp_plan *plan) {
     cudaError_t e = cudaDeviceSynchronize();
     plan_free(plan);
     return cuda_status(e);
+}
+
+fsp_status fsp_memory_trim(void) {
+    std::vector<DevPool> pools;
+    {
+        std::lock_guard<std::mutex> lk(g_pool_mu);
+        for (const auto &q : g_pools)
+            if (q.second.pool) pools.push_back(q.second);
+    }
+    fsp_status st = FSP_OK;
+    for (const DevPool &d : pools) {
+        DeviceScope scope(d.dev);
+        if (!scope.ok || pool_trim(d) != cudaSuccess) {
+            cudaGetLastError();
+            st = FSP_ECUDA;
+        }
+    }
+    return st;
 }
 
 fsp_status fsp_plan_set_timing(fsp_plan *plan, void *const *events, int nevents) {
@@ -2463,7 +2493,7 @@ void server_loop(fsp_server *v) {
                     break;
                 }
                 const size_t w1 = wb / 3;
-                if (cudaMalloc(&ws.W1, w1) != cudaSuccess || cudaMalloc(&ws.W2, 2 * w1) != cudaSuccess) {
+                if (device_malloc(&ws.W1, w1) != cudaSuccess || device_malloc(&ws.W2, 2 * w1) != cudaSuccess) {
                     cudaGetLastError();
                     if (ws.W1) cudaFree(ws.W1);
                     ws.W1 = nullptr;

@@ -140,7 +140,7 @@ fsp_status fsp_dist_create(fsp_dist **out, int N, double L, fsp_algo algo, fsp_d
     void **bufs[4] = {&d->W1, &d->W2, &d->V, &d->U};
     const size_t sizes[4] = {b1, b2, bv, bu};
     for (int i = 0; i < 4; ++i) {
-        if (cudaMalloc(bufs[i], sizes[i] ? sizes[i] : 16) != cudaSuccess) {
+        if (internal::device_malloc(bufs[i], sizes[i] ? sizes[i] : 16) != cudaSuccess) {
             cudaGetLastError();
             dist_free(d);
             return FSP_ENOMEM;

@@ -23,5 +23,8 @@ struct PlanView {
 fsp_status spectrum_plan_create(fsp_plan **out, int N, double L, fsp_algo algo, fsp_dtype dtype, cudaStream_t s);
 bool plan_view(const fsp_plan *p, PlanView *v);
 
+// cudaMalloc, tried again without the memory that the plan pool keeps unused.
+cudaError_t device_malloc(void **p, size_t bytes);
+
 }  // namespace internal
 }  // namespace fsp

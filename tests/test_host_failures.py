@@ -4,6 +4,7 @@ import ctypes
 import glob
 import os
 import subprocess
+import time
 
 import numpy as np
 import pytest
@@ -39,6 +40,10 @@ def fake(tmp_path_factory):
     L.fsp_batch_set_timeout.argtypes = [VP, d]
     L.fsp_batch_set_form.argtypes = [VP, i]
     L.fsp_batch_destroy.argtypes = [VP]
+    L.fsp_server_create.argtypes = [ctypes.POINTER(VP), ctypes.c_size_t, i]
+    L.fsp_server_submit.argtypes = [VP, i, d, i, i, VP, VP, ctypes.POINTER(ctypes.c_uint64)]
+    L.fsp_server_poll.argtypes = [VP, ctypes.c_uint64, ctypes.POINTER(i), ctypes.POINTER(d)]
+    L.fsp_server_destroy.argtypes = [VP]
     for f in ("fake_used", "fake_idle"):
         getattr(L, f).restype = ctypes.c_size_t
     L.fake_violations.restype = ctypes.c_long
@@ -157,3 +162,39 @@ def test_buffers_wait_for_their_own_device(fake):
     assert L.fsp_plan_destroy(on[0][1]) == OK
     assert L.fake_violations() == 0
     assert [L.fake_used(d) for d in (0, 1)] == used
+
+
+def test_kept_memory_is_within_reach(fake):
+    """What the library keeps of destroyed plans serves its other allocations
+    on a full device, and goes back on request."""
+    L = fake
+    L.fake_reset(2)  # as many as the tests before made pools on
+    used = L.fake_used(0)
+    assert L.fsp_memory_trim() == OK and L.fake_idle(0) == 0
+    for _ in range(3):
+        p = plan(L, 96, F32)
+        most = L.fake_used(0)
+        assert L.fsp_plan_destroy(p) == OK
+    kept = L.fake_idle(0)
+    assert L.fake_used(0) == used and 0 < most - used <= kept <= 1 << 30
+    # a server's workspace (N = 64: 7.9 MB), with half that much free
+    L.fake_capacity(used + kept + (4 << 20))
+    v, ticket, state = VP(), ctypes.c_uint64(), ctypes.c_int()
+    a = Arrays([64, 64], F32)
+    assert L.fsp_server_create(ctypes.byref(v), 1 << 30, 1) == OK
+    assert L.fsp_server_submit(v, 64, 1.0, HE, F32, a.ptrs[0], a.ptrs[1], ctypes.byref(ticket)) == OK
+    for _ in range(1000):
+        assert L.fsp_server_poll(v, ticket, ctypes.byref(state), None) == OK
+        if state.value >= 2:
+            break
+        time.sleep(0.01)
+    assert state.value == 2
+    assert L.fsp_server_destroy(v) == OK
+    assert L.fake_idle(0) > 0
+    # another allocator, which needs all of it
+    q = VP()
+    left = used + kept + (4 << 20) - L.fake_used(0)
+    assert L.cudaMalloc(ctypes.byref(q), ctypes.c_size_t(left)) != 0
+    assert L.fsp_memory_trim() == OK and L.fake_idle(0) == 0
+    assert L.cudaMalloc(ctypes.byref(q), ctypes.c_size_t(left)) == 0
+    assert L.cudaFree(q) == 0 and L.fake_violations() == 0
