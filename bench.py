@@ -495,7 +495,10 @@ def roofline(N, c, r, leg, dtype, hbm, hbm_kind):
     dur_s = float(leg["per_pass"][:, k].mean()) * 1e-3
     achieved = pb[k] / dur_s / 1e9
     name = PASS_NAMES[k] if dtype == "f32" else PASS_NAMES[k].replace("k_fast", "k_fx")
-    return {"bound": "hbm", "kernel": name, "achieved": round(achieved, 1), "peak": hbm,
+    # FP64 runs on the integer units: their multiply-add pipe is 68 % busy in
+    # P3 (profiles/p3_fx_f64_n256_ncu.md), DRAM 16 %
+    bound = "hbm" if dtype == "f32" else "integer multiply-add"
+    return {"bound": bound, "kernel": name, "achieved": round(achieved, 1), "peak": hbm,
             "unit": "GB/s", "frac": round(achieved / hbm, 4), "peak_kind": hbm_kind + " copy bandwidth",
             "traffic": recorded_traffic(dtype, N, k), "algorithmic_bytes": int(pb[k]),
             "pass_ms": [round(float(x), 4) for x in leg["per_pass"].mean(axis=0)],

@@ -385,7 +385,12 @@ fsp_status fsp_batch_destroy(fsp_batch *batch);
  * generic engine's row and column shapes of each distinct N (largest first),
  * timing graph replays of the batch itself; the winners are kept by the batch
  * and recorded in the tuning table (fsp_tuning_get).  Launches the batch many
- * times (it reads rho, overwrites phi); synchronises `stream`. */
+ * times (it reads rho, overwrites phi); synchronises `stream`.
+ *
+ * A batch that runs the specialised FP32 passes has no shapes to tune: it is
+ * timed on the generic engine for the table alone (the shapes serve batches
+ * with another size among them) and runs its own passes again afterwards.
+ * On failure the batch stays usable. */
 fsp_status fsp_batch_autotune(fsp_batch *batch, fsp_stream stream);
 /* create + launch + wait + destroy in one call. */
 fsp_status fsp_solve_batched(fsp_plan *const *plans, const void *const *rho, void *const *phi, int count,

@@ -427,7 +427,8 @@ class Batch:
         check(lib().fsp_batch_set_timeout(self._b, float(ms)), "fsp_batch_set_timeout")
 
     def autotune(self, stream=None):
-        """Tune the batch's tile shapes by timing its own launches."""
+        """Tune the generic engine's tile shapes on this batch (for the tuning
+        table alone where the batch runs the specialised FP32 passes)."""
         check(lib().fsp_batch_autotune(self._b, _stream_handle(stream)), "fsp_batch_autotune")
 
     def inject_stall(self):

@@ -480,8 +480,8 @@ FSP_CFGX(384, 24, 8, 8, 6, 8)
 FSP_CFGX(512, 8, 4, 8, 8, 8)
 FSP_CFGX(1024, 16, 4, 16, 8, 8)
 #undef FSP_CFGX
-// Rows: lengths 64 and 256 run faster in two stages (P1 / P5 at N = 256 0.155 /
-// 0.151 ms with 16*16, 0.163 / 0.161 with 8*4*8)
+// Rows: lengths 64 and 256 run faster in two stages (P1 / P5 at N = 256 0.161 /
+// 0.152 ms with 16*16, 0.166 / 0.162 with 8*4*8)
 template <int N> struct RowX : CfgX<N> {};
 template <> struct RowX<64> {
     static constexpr int V = 8, L = 16, R1 = 8, R2 = 8, R3 = 1;
@@ -490,8 +490,8 @@ template <> struct RowX<256> {
     static constexpr int V = 16, L = 8, R1 = 16, R2 = 16, R3 = 1;
 };
 // CTAs per SM the registers must allow.  With 8 values per thread 24 warps for
-// P3 (80 registers, a few spilled: 1.055 ms at N = 256, 1.063 with 32 warps,
-// 1.14 with 16) and 32 for P2 and P4 (0.266 / 0.255 ms, 0.273 / 0.274 with
+// P3 (80 registers, a few spilled: 1.051 ms at N = 256, 1.071 with 32 warps,
+// 1.149 with 16) and 32 for P2 and P4 (0.267 / 0.256 ms, 0.275 / 0.285 with
 // 24); fewer where a thread holds more.
 template <int n, int MODE> constexpr int fx_minb() {
     constexpr int th = CfgX<n>::L * (n / CfgX<n>::V), V = CfgX<n>::V;

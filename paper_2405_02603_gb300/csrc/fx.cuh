@@ -88,9 +88,9 @@ __device__ __forceinline__ cfx fx_cmul(long long x, long long y, int rh, int rl,
     const long long q = fx_mad(xh, il, fx_mad(xl, ih, fx_mad(yh, rl, fx_mad(yl, rh, kFxHalf))));
     return cfx{fx(fx_mad(xh, rh, fx_mad(yh, uh, fx_high(p))), 0), fx(fx_mad(xh, ih, fx_mad(yh, rh, fx_high(q))), 0)};
 }
-// Constants of modulus < 1, with 63 fraction bits: w 2 wraps to (w - k) 2^64, k
-// one of -1, 0, 1 (fx_whole), so that w a = k a + a (w - k) 2^64 / 2^64 and a need
-// not be doubled.
+// Constants w of modulus < 1, with 63 fraction bits: twice w 2^63 wraps to
+// (w - k) 2^64, k one of -1, 0, 1 (fx_whole), so w a = k a + a ((w - k) 2^64) / 2^64
+// and a need not be doubled.
 __host__ __device__ constexpr long long fx_twice(long long c) { return (long long)((unsigned long long)c << 1); }
 __host__ __device__ constexpr int fx_whole(long long c) { return c >= 1LL << 62 ? 1 : c < -(1LL << 62) ? -1 : 0; }
 // constant c times a, |a| < 2^63
