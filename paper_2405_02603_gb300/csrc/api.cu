@@ -657,6 +657,9 @@ struct fsp_plan {
     void *tw_y = nullptr, *tw_z = nullptr;
     cudaEvent_t ev[6] = {};
     bool timing = false;
+    // FP64 plans hold S divided by 2^s_exp and SF by 2^f_exp, and P5 multiplies
+    // by that: 0 in ordinary boxes (fx_line.cuh: the product with S)
+    int s_exp = 0, f_exp = 0;
     bool guarded = false;  // FSP_CHECK_BOUNDS=1 at creation: buffers with guard bands
     size_t bytes = 0;
     double precompute_ms = 0;
@@ -667,6 +670,22 @@ namespace {
 bool plan_live(const fsp_plan *p) {
     std::lock_guard<std::mutex> lk(g_mu);
     return p && g_plans.count(p) && p->magic == kMagic;
+}
+
+// The order of a spectrum as a power of two, 0 within 2^+-50.
+int order_of(double x) {
+    const int e = x > 0.0 && std::isfinite(x) ? std::ilogb(x) : 0;
+    return std::abs(e) < 50 ? 0 : std::min(1000, std::max(-1000, e));
+}
+// s_exp and f_exp of an FP64 plan: h^3 / (8 n_x n_y n_z) times the box's integral of
+// 1 / 4 pi r (L^2 within a few octaves; Hockney-Eastwood also has its value at the
+// origin, which does not scale) or of its derivative (L).
+void spectrum_exps(fsp_plan *p, const int *n, const double *h) {
+    if (!is_f64(p->dtype)) return;
+    double L = 0.0, per = 0.125, at0 = p->algo == FSP_HE ? 0.08 : 0.0;
+    for (int a = 0; a < 3; ++a) L = std::max(L, n[a] * h[a]), per /= n[a], at0 *= h[a];
+    p->s_exp = order_of(std::max(L * L, at0) * per);
+    p->f_exp = order_of(L * per);
 }
 
 // grid points of a plan's source / result
@@ -729,6 +748,7 @@ cudaError_t enqueue_solve_fast(const fsp_plan *p, const void *rho, void *phi, vo
     cudaError_t e;
     auto mark = [&](int i) { return p->timing ? cudaEventRecord(p->ev[i], s) : cudaSuccess; };
     fast::RowArgs r{};
+    r.exp = p->s_exp;
     r.x = rho, r.c = W1, r.x_row = N, r.c_row = P, r.nrows = N * N, r.tw = p->tw_n, r.tw2 = p->tw_2n;
     fast::ColArgs a{};
     a.tw = p->tw_2n, a.nlines = N + 1;
@@ -772,6 +792,7 @@ cudaError_t enqueue_solve_generic(const fsp_plan *p, const void *rho, void *phi,
     // P1: pad + x-R2C (rows of rho -> W1[z][y][kx])
     if ((e = mark(0)) != cudaSuccess) return e;
     RowsArgs r{};
+    r.exp = p->s_exp;
     r.x = rho, r.c = W1, r.x_row = N, r.c_row = P, r.N = N, r.nrows = N * N;
     r.lgL = p->row.lgL, r.tpl = p->row.tpl, r.st = p->row.st, r.tw = p->tw_n, r.tw2 = p->tw_2n;
     if ((e = launch_r2c_rows<T>(r, s)) != cudaSuccess) return e;
@@ -855,7 +876,7 @@ cudaError_t enqueue_field_fast(const fsp_plan *p, const void *rho, void *const o
         b.in = p->W3, b.out = p->W1, b.odd = 0;
         b.in_pos = P, b.in_batch = 2LL * N * P, b.out_pos = P, b.out_batch = (long long)N * P;
         if ((e = fast::p4<T>(N, b, N, s)) != cudaSuccess) return e;
-        r.x = out[c];
+        r.x = out[c], r.exp = c == 3 ? p->s_exp : p->f_exp;
         if ((e = fast::p5<T>(N, r, s)) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -891,7 +912,7 @@ cudaError_t enqueue_field_generic(const fsp_plan *p, const void *rho, void *cons
         b.out_pos = P, b.out_batch = (long long)N * P;
         b.n_in = 2 * N, b.n_out = N, b.nbatch = N;
         if ((e = launch_lines<T, IN_CPLX, OUT_CPLX, M_INV>(b, s)) != cudaSuccess) return e;
-        r.x = out[c];
+        r.x = out[c], r.exp = c == 3 ? p->s_exp : p->f_exp;
         if ((e = launch_c2r_rows<T>(r, s)) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -927,7 +948,7 @@ cudaError_t enqueue_field_aniso(const fsp_plan *p, const void *rho, void *const 
             b.tw = p->tw_y, b.in = p->W3, b.out = p->W1, b.odd = 0;
             b.in_pos = P, b.in_batch = 2LL * ny * P, b.out_pos = P, b.out_batch = (long long)ny * P;
             if ((e = fast::col_rg<T>(fast::COL_INV, 2 * ny, b, nz, s)) != cudaSuccess) return e;
-            r.x = out[c];
+            r.x = out[c], r.exp = c == 3 ? p->s_exp : p->f_exp;
             if ((e = fast::p5<T>(nx, r, s)) != cudaSuccess) return e;
         }
         return cudaSuccess;
@@ -960,7 +981,7 @@ cudaError_t enqueue_field_aniso(const fsp_plan *p, const void *rho, void *const 
             b.out_pos = P, b.out_batch = (long long)ny * P;
             b.n_in = 2 * ny, b.n_out = ny, b.nbatch = nz;
             if ((e = launch_lines<T, IN_CPLX, OUT_CPLX, M_INV>(b, s)) != cudaSuccess) return e;
-            r.x = out[c];
+            r.x = out[c], r.exp = c == 3 ? p->s_exp : p->f_exp;
             if ((e = launch_c2r_rows<T>(r, s)) != cudaSuccess) return e;
         }
         return cudaSuccess;
@@ -989,6 +1010,7 @@ cudaError_t enqueue_solve_aniso(const fsp_plan *p, const void *rho, void *phi, v
     auto mark = [&](int i) { return p->timing ? cudaEventRecord(p->ev[i], s) : cudaSuccess; };
     if ((e = mark(0)) != cudaSuccess) return e;
     RowsArgs r{};
+    r.exp = p->s_exp;
     r.x = rho, r.c = W1, r.x_row = nx, r.c_row = P, r.N = nx, r.nrows = ny * nz;
     r.lgL = p->row.lgL, r.tpl = p->row.tpl, r.st = p->row.st, r.tw = p->tw_n, r.tw2 = p->tw_2n;
     if ((e = launch_r2c_rows<T>(r, s)) != cudaSuccess) return e;
@@ -1029,6 +1051,7 @@ cudaError_t enqueue_solve_aniso_fast(const fsp_plan *p, const void *rho, void *p
     cudaError_t e;
     auto mark = [&](int i) { return p->timing ? cudaEventRecord(p->ev[i], s) : cudaSuccess; };
     fast::RowArgs r{};
+    r.exp = p->s_exp;
     r.x = rho, r.c = W1, r.x_row = nx, r.c_row = P, r.nrows = ny * nz, r.tw = p->tw_n, r.tw2 = p->tw_2n;
     if ((e = mark(0)) != cudaSuccess) return e;
     if ((e = fast::p1<T>(nx, r, s)) != cudaSuccess) return e;
@@ -1090,9 +1113,10 @@ const char *fsp_status_str(fsp_status s) {
 
 namespace {
 // s_host: null to compute the spectrum (Sec. 2.2-2.4), else (N+1)^3 doubles
-// of a stored one (the octant fsp_plan_spectrum writes, already scaled)
+// of a stored one (the octant fsp_plan_spectrum writes, already scaled), the
+// largest of them s_max in modulus
 fsp_status plan_create_impl(fsp_plan **out, int N, double L, double h, fsp_algo algo, fsp_dtype dtype,
-                            fsp_stream stream, bool with_workspace, const double *s_host = nullptr) {
+                            fsp_stream stream, bool with_workspace, const double *s_host = nullptr, double s_max = 0.0) {
     if (!out) return FSP_EINVAL;
     *out = nullptr;
     fsp_status st = validate_size(N, L, algo);
@@ -1110,6 +1134,11 @@ fsp_status plan_create_impl(fsp_plan **out, int N, double L, double h, fsp_algo 
     p->N = N, p->L = L, p->h = L / N, p->algo = algo, p->dtype = dtype;
     p->rsize = dtype == FSP_F32_MIXED ? 4 : 8;  // caller's reals
     p->P = ((N + 1) + 15) / 16 * 16;
+    {
+        const int n3[3] = {N, N, N};
+        const double h3[3] = {p->h, p->h, p->h};
+        spectrum_exps(p, n3, h3);
+    }
     const size_t csize = 2 * p->rsize;
     // tiles: rows (length-N FFT, N+1 positions), columns (length 2N)
     int row_lgL = dtype == FSP_F32_MIXED ? 4 : 3, col_lgL = dtype == FSP_F32_MIXED ? 4 : 3;
@@ -1182,6 +1211,8 @@ fsp_status plan_create_impl(fsp_plan **out, int N, double L, double h, fsp_algo 
                 cudaSuccess)
                 return fail(FSP_ECUDA);
             scale = 1.0;
+            // a spectrum of another order than the box's
+            if (is_f64(dtype) && s_max > 0.0 && std::abs(std::ilogb(s_max) - p->s_exp) >= 60) p->s_exp = order_of(s_max);
         } else {
             if ((st = enqueue_kernel_T(N, L, algo, (double *)Td.p, s, tmp)) != FSP_OK) return fail(st);
             if ((st = enqueue_dct_spectrum(N, (double *)Td.p, s, tw)) != FSP_OK) return fail(st);
@@ -1192,7 +1223,7 @@ fsp_status plan_create_impl(fsp_plan **out, int N, double L, double h, fsp_algo 
             mx *= std::fabs(scale);
             if (!(mx >= kDfMinS && mx <= kDfMaxS)) return fail(FSP_EUNSUPPORTED);
         }
-        e = is_f64(dtype) ? launch_store_S<double>((double *)Td.p, p->S, N, p->P, scale, s)
+        e = is_f64(dtype) ? launch_store_S<double>((double *)Td.p, p->S, N, p->P, std::ldexp(scale, -p->s_exp), s)
                           : launch_store_S<float>((double *)Td.p, p->S, N, p->P, scale, s);
         if (e != cudaSuccess) return fail(FSP_ECUDA);
         if (cudaStreamSynchronize(s) != cudaSuccess) return fail(FSP_ECUDA);
@@ -1227,7 +1258,7 @@ fsp_status spectrum_plan_create(fsp_plan **out, int N, double L, fsp_algo algo, 
 
 bool plan_view(const fsp_plan *p, PlanView *v) {
     if (!plan_live(p) || !v || p->aniso) return false;
-    v->N = p->N, v->P = p->P, v->device = p->device, v->dtype = p->dtype, v->rsize = p->rsize;
+    v->N = p->N, v->P = p->P, v->device = p->device, v->s_exp = p->s_exp, v->dtype = p->dtype, v->rsize = p->rsize;
     v->S = p->S, v->tw_n = p->tw_n, v->tw_2n = p->tw_2n, v->row = p->row, v->col = p->col;
     return true;
 }
@@ -1247,12 +1278,15 @@ fsp_status fsp_plan_create_from_spectrum(fsp_plan **out, int N, double L, fsp_al
     if (!out) return FSP_EINVAL;
     *out = nullptr;
     if (!s_host) return FSP_EINVAL;
+    double s_max = 0.0;
     if (N >= 2 && N <= kMaxN) {  // every value finite (a truncated or corrupt file shows here first)
         const size_t tot = (size_t)(N + 1) * (N + 1) * (N + 1);
-        for (size_t i = 0; i < tot; ++i)
+        for (size_t i = 0; i < tot; ++i) {
             if (!std::isfinite(s_host[i])) return FSP_EINVAL;
+            s_max = std::max(s_max, std::fabs(s_host[i]));
+        }
     }
-    return plan_create_impl(out, N, L, L / N, algo, dtype, stream, true, s_host);
+    return plan_create_impl(out, N, L, L / N, algo, dtype, stream, true, s_host, s_max);
 }
 
 fsp_status fsp_plan_create_aniso(fsp_plan **out, int nx, int ny, int nz, double hx, double hy, double hz,
@@ -1302,6 +1336,7 @@ fsp_status fsp_plan_create_aniso(fsp_plan **out, int nx, int ny, int nz, double 
     p->fast = fast_ok;
     for (int a = 0; a < 3; ++a) p->n3[a] = nn[a], p->h3[a] = hh[a];
     p->N = nx, p->L = nx * hx, p->h = hx, p->algo = algo, p->dtype = dtype;
+    spectrum_exps(p, nn, hh);
     p->rsize = dtype == FSP_F32_MIXED ? 4 : 8;
     p->P = ((nx + 1) + 15) / 16 * 16;
     const size_t csize = 2 * p->rsize;
@@ -1361,7 +1396,7 @@ fsp_status fsp_plan_create_aniso(fsp_plan **out, int nx, int ny, int nz, double 
             mx *= std::fabs(scale);
             if (!(mx >= kDfMinS && mx <= kDfMaxS)) return fail(FSP_EUNSUPPORTED);
         }
-        e = is_f64(dtype) ? launch_store_S3<double>((double *)Td.p, p->S, nx + 1, rows, p->P, scale, s)
+        e = is_f64(dtype) ? launch_store_S3<double>((double *)Td.p, p->S, nx + 1, rows, p->P, std::ldexp(scale, -p->s_exp), s)
                           : launch_store_S3<float>((double *)Td.p, p->S, nx + 1, rows, p->P, scale, s);
         if (e != cudaSuccess) return fail(FSP_ECUDA);
         if (cudaStreamSynchronize(s) != cudaSuccess) return fail(FSP_ECUDA);
@@ -1432,7 +1467,7 @@ fsp_status fsp_plan_field_init(fsp_plan *plan, fsp_stream stream) {
             return st;
         }
         cudaError_t e =
-            is_f64(plan->dtype) ? launch_store_S3<double>((double *)Fd.p, bs[axis].p, kx, rows, plan->P, scale, s)
+            is_f64(plan->dtype) ? launch_store_S3<double>((double *)Fd.p, bs[axis].p, kx, rows, plan->P, std::ldexp(scale, -plan->f_exp), s)
                                         : launch_store_S3<float>((double *)Fd.p, bs[axis].p, kx, rows, plan->P, scale, s);
         if (cudaStreamSynchronize(s) != cudaSuccess || e != cudaSuccess) return FSP_ECUDA;
     }
@@ -1663,6 +1698,7 @@ double fsp_plan_precompute_ms(const fsp_plan *plan) { return plan_live(plan) ? p
 fsp_status fsp_plan_spectrum(const fsp_plan *plan, double *s_host) {
     if (!plan_live(plan) || !s_host) return FSP_EINVAL;
     StreamScope stream_scope(nullptr);
+    const double back = std::ldexp(1.0, plan->s_exp);
     if (plan->aniso) {
         const int kx = plan->n3[0] + 1;
         const long long rows = (long long)(plan->n3[1] + 1) * (plan->n3[2] + 1);
@@ -1670,8 +1706,8 @@ fsp_status fsp_plan_spectrum(const fsp_plan *plan, double *s_host) {
         DevBuf d;
         fsp_status st = alloc_or_nomem(d, sizeof(double) * tot);
         if (st != FSP_OK) return st;
-        cudaError_t e = is_f64(plan->dtype) ? launch_load_S3<double>(plan->S, (double *)d.p, kx, rows, plan->P, 0)
-                                                    : launch_load_S3<float>(plan->S, (double *)d.p, kx, rows, plan->P, 0);
+        cudaError_t e = is_f64(plan->dtype) ? launch_load_S3<double>(plan->S, (double *)d.p, kx, rows, plan->P, back, 0)
+                                                    : launch_load_S3<float>(plan->S, (double *)d.p, kx, rows, plan->P, back, 0);
         if (e != cudaSuccess) return FSP_ECUDA;
         return cuda_status(cudaMemcpy(s_host, d.p, sizeof(double) * tot, cudaMemcpyDeviceToHost));
     }
@@ -1679,8 +1715,8 @@ fsp_status fsp_plan_spectrum(const fsp_plan *plan, double *s_host) {
     DevBuf d;
     fsp_status st = alloc_or_nomem(d, sizeof(double) * tot);
     if (st != FSP_OK) return st;
-    cudaError_t e = is_f64(plan->dtype) ? launch_load_S<double>(plan->S, (double *)d.p, plan->N, plan->P, 0)
-                                                : launch_load_S<float>(plan->S, (double *)d.p, plan->N, plan->P, 0);
+    cudaError_t e = is_f64(plan->dtype) ? launch_load_S<double>(plan->S, (double *)d.p, plan->N, plan->P, back, 0)
+                                                : launch_load_S<float>(plan->S, (double *)d.p, plan->N, plan->P, back, 0);
     if (e != cudaSuccess) return FSP_ECUDA;
     return cuda_status(cudaMemcpy(s_host, d.p, sizeof(double) * tot, cudaMemcpyDeviceToHost));
 }
@@ -1816,7 +1852,7 @@ BatchSolve batch_solve_of(const fsp_plan *p, const void *rho, void *phi, const T
     r.lgL = row.lgL, r.tpl = row.tpl, r.st = row.st, r.tw = p->tw_n, r.tw2 = p->tw_2n;
     b.r1 = r, b.r5 = r;
     b.r1.x = rho;
-    b.r5.x = phi;
+    b.r5.x = phi, b.r5.exp = p->s_exp;
     LinesArgs a{};
     a.st = col.st, a.tpl = col.tpl, a.lgL = col.lgL, a.tw = p->tw_2n;
     a.nlines = N + 1;

@@ -247,7 +247,7 @@ cudaError_t dist_backward(fsp_dist *d, const void *const *recv, void *phi, cudaS
             return e;
     }
     RowsArgs r{};  // P5: x-C2R, crop x, W1 rows -> phi slab
-    r.x = phi, r.c = d->W1, r.x_row = N, r.c_row = P, r.N = N, r.nrows = (int)(nz * N);
+    r.x = phi, r.c = d->W1, r.x_row = N, r.c_row = P, r.N = N, r.nrows = (int)(nz * N), r.exp = v.s_exp;
     r.lgL = v.row.lgL, r.tpl = v.row.tpl, r.st = v.row.st, r.tw = v.tw_n, r.tw2 = v.tw_2n;
     if (nz > 0 && (e = launch_c2r_rows<T>(r, s)) != cudaSuccess) return e;
     return cudaSuccess;

@@ -35,6 +35,7 @@ struct RowArgs {
     int nrows;
     const void *tw;   // roots of length N
     const void *tw2;  // roots of length 2N
+    int exp;          // FP64 P5: results times 2^exp (the plan's spectrum is divided by it)
 };
 
 enum ColMode { COL_FWD = 0, COL_INV = 1, COL_FMI = 2, COL_FMO = 3 };

@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(L *(n / V), MINB) k_fx_col(const ColArgs a) {
                 constexpr int r = decltype(rc)::value, i = k * RL + r, c = k * TPL + r * (n / RL);
                 const int p = t + c, fz = p <= N ? p : n - p;
                 const cfx q = fx_mul_s(v[i], __ldg(Sy + (long long)fz * S_POS), ke,
-                                       MODE == COL_FMO ? flip_b ^ (p > N ? flip_z : 0) : 0, near);
+                                       MODE == COL_FMO ? flip_b ^ (p > N ? flip_z : 0) : 0, eS > -900);
                 v[i] = MODE == COL_FMI ? q : cfx{q.y, -q.x};
             });
         });
@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(L *(N / V)) k_fx_c2r(const RowArgs a) {
     Fst<+1, N, V, L>::template compute<R1, 1, false, false>(v, t, tw);
     fx_rest<+1, N, V, L, R1, R2, R3, true>(v, buf, t, l, tw, true);
     __syncthreads();
-    const FxOut<true, true> out(2 * NT + 2 - sc.ke, sc.bad);
+    const FxOut<true, true> out(2 * NT + 2 - sc.ke + a.exp, sc.bad);
 #pragma unroll
     for (int k = 0; k < V / RL; ++k)
 #pragma unroll

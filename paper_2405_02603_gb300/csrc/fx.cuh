@@ -156,9 +156,11 @@ template <int D, int m> __device__ __forceinline__ cfx fx_w32(cfx a) {
 // ------------------------------------------------ doubles <-> a line's scale --
 // upper 32 bits of |x|
 __device__ __forceinline__ int fx_habs(double x) { return __double2hiint(x) & 0x7fffffff; }
-// |x| as a float, from its upper word (truncated, relative error < 2^-20), for
-// |x| < 2^127; 0 below 2^-126
-__device__ __forceinline__ float fx_fabs(int h) { return __uint_as_float((unsigned)max(h, 896 << 20) * 8u - (896u << 23)); }
+// |x| 2^-k as a float, from the upper word of |x| (truncated, relative error <
+// 2^-20), for |x| 2^-k < 2^127; 0 below 2^-126.  -1023 <= k <= 1024.
+__device__ __forceinline__ float fx_fabs(int h, int k = 0) {
+    return __uint_as_float((unsigned)max(h, (896 + k) * 0x100000) * 8u - ((unsigned)(896 + k) << 23));
+}
 // ceil(log2 x) of a positive float
 __device__ __forceinline__ int fx_clog2(float x) { return ((__float_as_int(x) + 0x7fffff) >> 23) - 127; }
 

@@ -15,12 +15,12 @@ __host__ __device__ constexpr int fx_grow(int R) {
 __device__ __forceinline__ cfx fx_raw(double2 q) {
     return cfx{fx(__double_as_longlong(q.x), 0), fx(__double_as_longlong(q.y), 0)};
 }
-// adds its modulus (within sqrt 2) to s, and the upper word of its larger
-// component to the maximum h
-__device__ __forceinline__ void fx_bound(const cfx &v, float &s, int &h) {
+// adds its modulus (within sqrt 2), in units of 2^k, to s, and the upper word of
+// its larger component to the maximum h
+__device__ __forceinline__ void fx_bound(const cfx &v, float &s, int &h, int k = 0) {
     const int hx = fx_habs(__longlong_as_double(v.x.v)), hy = fx_habs(__longlong_as_double(v.y.v));
     const int m = max(hx, hy);
-    s += fx_fabs(m);
+    s += fx_fabs(m, k);
     h = max(h, m);
 }
 
@@ -32,8 +32,12 @@ struct FxScale {
 };
 // components of a line are below 2^em, hmax the largest upper word
 __device__ __forceinline__ int fx_em(int hmax) { return max(hmax >> 20, 1) - 1022; }
-// the range of em in which fx_fabs, fx_of and fx_of_p hold
-__device__ __forceinline__ bool fx_far(int em) { return em < -60 || em > 90; }
+// outside the range of em in which sums of fx_fabs, fx_of and fx_of_p hold: below,
+// values that count as zero would reach the 1-norm's last bits; above, it could
+// overflow a float.  (Sources of 1e-30 .. 1e33: FP64 plans keep their spectra
+// near 1.)  A line outside has the scale of its largest component alone in the
+// specialised passes, at most 4 bits below the one of its 1-norm.
+__device__ __forceinline__ bool fx_far(int em) { return em < -100 || em > 112; }
 
 // ---- the scale of a line with a runtime schedule (kernels_impl.cuh)
 // s <= 2^em * (some 2^12) in units of 2^(em - 16), rounded up; |em| < 100
@@ -92,21 +96,30 @@ template <bool PX, bool PY> struct FxOut {
 //   r = 1022 - ke - es
 // (S is shifted rather than the products: one value, and its dropped bits are
 // worth less than a unit of the result).
-__device__ __forceinline__ void fx_bound_mul(const cfx &v, double s, float &s2, float &m2, int &hS) {
+//
+// The bounds are floats, which hold for |S| 2^-k in (2^-80, 2^80); a line outside
+// has the bounds of the largest S and the largest possible v alone, 4 (N = 32)
+// to 11 bits (N = 135) wider.  S scales with the square of the box (2^-100 in
+// boxes of 1e-12, 2^114 in boxes of 1e20), so FP64 plans hold it divided by a
+// power of two that P5 gives back, and k = 0 does.  A caller's bare spectrum,
+// which only the generic engine meets, has the exponent of S(1, 1, 1) as its k:
+// close to the largest of a potential's.
+__device__ __forceinline__ int fx_base(double s) { return max(fx_habs(s) >> 20, 1) - 1023; }
+__device__ __forceinline__ void fx_bound_mul(const cfx &v, double s, float &s2, float &m2, int &hS, int k = 0) {
     const int hs = fx_habs(s);
     // |v| <= f 2^32
     const float f = (float)(abs((int)(v.x.v >> 32)) + abs((int)(v.y.v >> 32)) + 2);
-    const float q = f * fx_fabs(hs);
+    const float q = f * fx_fabs(hs, k);
     s2 += q, m2 = fmaxf(m2, q), hS = max(hS, hs);
 }
 // exponent of the largest |S|, and whether the float bounds hold for it
 __device__ __forceinline__ int fx_es(int hS) { return (hS >> 20) - 1022; }
-__device__ __forceinline__ bool fx_near(int eS) { return eS > -90 && eS < 80; }
-// neg: -1 to negate S; near: as fx_near (else S may be zero or subnormal at a
-// scale where that is not simply a zero product)
-__device__ __forceinline__ cfx fx_mul_s(const cfx &v, double s, int ke, int neg, bool near) {
+__device__ __forceinline__ bool fx_near(int eS, int k = 0) { return eS - k > -80 && eS - k < 80; }
+// neg: -1 to negate S; normal: the largest |S| is above 2^-900, so that a
+// subnormal one gives a zero product whatever its leading bit
+__device__ __forceinline__ cfx fx_mul_s(const cfx &v, double s, int ke, int neg, bool normal) {
     const int hi = __double2hiint(s), e = (hi >> 20) & 0x7ff, sh = 1022 - ke - max(e, 1);
-    const int one = near || e != 0 ? 0x100000 : 0;
+    const int one = normal || e != 0 ? 0x100000 : 0;
     const unsigned long long m = ((unsigned long long)((hi & 0xfffff) | one) << 32) | (unsigned)__double2loint(s);
     const long long mr = (long long)(m << 9) >> min(max(sh, 0), 63), sg = (hi >> 31) ^ neg;
     const long long w = (mr ^ sg) - sg;

@@ -171,11 +171,11 @@ template <typename T> __global__ void k_store_S(const double *Sd, T *S, int kx, 
 }
 
 // S (pitch P, type T) -> dense rows of kx doubles
-template <typename T> __global__ void k_load_S(const T *S, double *Sd, int kx, long long rows, int P) {
+template <typename T> __global__ void k_load_S(const T *S, double *Sd, int kx, long long rows, int P, double scale) {
     const long long tot = (long long)kx * rows;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < tot; i += (long long)gridDim.x * blockDim.x) {
         const int x = (int)(i % kx);
-        Sd[i] = (double)S[(i / kx) * P + x];
+        Sd[i] = (double)S[(i / kx) * P + x] * scale;
     }
 }
 
@@ -248,8 +248,9 @@ cudaError_t launch_store_S3(const double *Sd, void *S, int kx, long long rows, i
     return cudaGetLastError();
 }
 
-template <typename T> cudaError_t launch_load_S3(const void *S, double *Sd, int kx, long long rows, int P, cudaStream_t s) {
-    k_load_S<T><<<grid_for((long long)kx * rows), 256, 0, s>>>(reinterpret_cast<const T *>(S), Sd, kx, rows, P);
+template <typename T>
+cudaError_t launch_load_S3(const void *S, double *Sd, int kx, long long rows, int P, double scale, cudaStream_t s) {
+    k_load_S<T><<<grid_for((long long)kx * rows), 256, 0, s>>>(reinterpret_cast<const T *>(S), Sd, kx, rows, P, scale);
     return cudaGetLastError();
 }
 
@@ -257,8 +258,8 @@ template <typename T> cudaError_t launch_store_S(const double *Sd, void *S, int 
     return launch_store_S3<T>(Sd, S, N + 1, (long long)(N + 1) * (N + 1), P, scale, s);
 }
 
-template <typename T> cudaError_t launch_load_S(const void *S, double *Sd, int N, int P, cudaStream_t s) {
-    return launch_load_S3<T>(S, Sd, N + 1, (long long)(N + 1) * (N + 1), P, s);
+template <typename T> cudaError_t launch_load_S(const void *S, double *Sd, int N, int P, double scale, cudaStream_t s) {
+    return launch_load_S3<T>(S, Sd, N + 1, (long long)(N + 1) * (N + 1), P, scale, s);
 }
 
 cudaError_t launch_he_T3(double *T, const int *n, const double *h, cudaStream_t s) {
@@ -286,11 +287,11 @@ cudaError_t launch_vg_sample_full3(void *g, const int *n, const double *h, doubl
 
 template cudaError_t launch_store_S<float>(const double *, void *, int, int, double, cudaStream_t);
 template cudaError_t launch_store_S<double>(const double *, void *, int, int, double, cudaStream_t);
-template cudaError_t launch_load_S<float>(const void *, double *, int, int, cudaStream_t);
-template cudaError_t launch_load_S<double>(const void *, double *, int, int, cudaStream_t);
+template cudaError_t launch_load_S<float>(const void *, double *, int, int, double, cudaStream_t);
+template cudaError_t launch_load_S<double>(const void *, double *, int, int, double, cudaStream_t);
 template cudaError_t launch_store_S3<float>(const double *, void *, int, long long, int, double, cudaStream_t);
 template cudaError_t launch_store_S3<double>(const double *, void *, int, long long, int, double, cudaStream_t);
-template cudaError_t launch_load_S3<float>(const void *, double *, int, long long, int, cudaStream_t);
-template cudaError_t launch_load_S3<double>(const void *, double *, int, long long, int, cudaStream_t);
+template cudaError_t launch_load_S3<float>(const void *, double *, int, long long, int, double, cudaStream_t);
+template cudaError_t launch_load_S3<double>(const void *, double *, int, long long, int, double, cudaStream_t);
 
 }  // namespace fsp

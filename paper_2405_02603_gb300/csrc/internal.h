@@ -14,7 +14,8 @@ struct PlanView {
     int N = 0, P = 0, device = 0;
     fsp_dtype dtype = FSP_F64;
     size_t rsize = 8;                      // bytes per real of the solve's arrays
-    const void *S = nullptr;               // S[q_z][q_y][q_x], pitch P, (N+1)^2 rows
+    const void *S = nullptr;               // S[q_z][q_y][q_x] / 2^s_exp, pitch P, (N+1)^2 rows
+    int s_exp = 0;                         // FP64: P5 multiplies by 2^s_exp
     const void *tw_n = nullptr, *tw_2n = nullptr;  // roots of length N and 2N
     TileCfg row, col;                      // generic engine: rows (length N), columns (length 2N)
 };

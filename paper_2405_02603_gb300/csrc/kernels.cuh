@@ -61,6 +61,7 @@ struct RowsArgs {
     Stages st;       // length N
     const void *tw;  // length-N roots
     const void *tw2; // length-2N roots
+    int exp;         // FP64 C2R: results times 2^exp (the plan's spectrum is divided by it)
 };
 
 inline int smem_pitch(int lgL) { return (1 << lgL) + 1; }

@@ -68,9 +68,16 @@ __device__ __forceinline__ FxScale tile_scale(cfx *buf, int ld, int np, const St
     const int em = fx_em(h);
     FxScale sc;
     sc.any = fx_far(em), sc.bad = (h >> 20) == 0x7ff;
-    if (act && !sc.any) atomicAdd(&q.sum[l], tile_units(s, em));
+    const bool sum = h != 0 && !sc.bad;  // neither a zero line nor an infinite one
+    if (act && sum) {
+        if (sc.any) {  // the 1-norm in units of 2^em: as it is, no float holds it
+            s = 0.f;
+            for (int p = sub; p < np; p += tpl) fx_bound(buf[p * ld + l], s, h, em);
+        }
+        atomicAdd(&q.sum[l], tile_units(s, sc.any ? 0 : em));
+    }
     __syncthreads();
-    const int eL = sc.any ? em + tile_log2(st) : em - 16 + fx_clog2(1.5f * (float)q.sum[l] + 1e-30f);
+    const int eL = sum ? em - 16 + fx_clog2(1.5f * (float)q.sum[l] + 1e-30f) : em + tile_log2(st);
     sc.ke = tile_ke(st, em, eL, B);
     if (act)
         for (int p = sub; p < np; p += tpl) buf[p * ld + l] = fx_conv<true, false>(buf[p * ld + l], sc);
@@ -231,20 +238,21 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
             // as k_fx_col: bounds of the products, then the products at the
             // scale of the inverse
             const double *Sl = S + (long long)fy * a.s_batch + line0 + l;
+            const int kS = fx_base(S[a.s_pos + a.s_batch + 1]);
             float s2 = 0.f, m2 = 0.f;
             int hS = 0;
             if (act) {
                 for (int p = sub; p < n; p += a.tpl)
-                    fx_bound_mul(buf[p * ld + l], Sl[(long long)(p <= a.half ? p : h2 - p) * a.s_pos], s2, m2, hS);
+                    fx_bound_mul(buf[p * ld + l], Sl[(long long)(p <= a.half ? p : h2 - p) * a.s_pos], s2, m2, hS, kS);
                 atomicMax(&tl.hS[l], hS);
                 atomicMax(&tl.mmax[l], __float_as_int(m2));
             }
             __syncthreads();
             const int eS = fx_es(tl.hS[l]);
-            const bool near = fx_near(eS), bad = sc.bad || eS == 1025;
-            // products' moduli are below 2^em (near: in units of 2^32)
+            const bool near = fx_near(eS, kS), bad = sc.bad || eS == 1025;
+            // products' moduli are below 2^em (near: in units of 2^(32 + kS))
             const int ef = fx_clog2(1.1f * __int_as_float(tl.mmax[l]));
-            const int em = near ? ef + 32 : 61 + eS;
+            const int em = near ? ef + 32 + kS : 61 + eS;
             if (act && near) atomicAdd(&tl.sum2[l], tile_units(s2, ef));
             __syncthreads();
             const int eL = near ? em - 16 + fx_clog2(1.1f * (float)tl.sum2[l] + 1e-30f) : em + tile_log2(a.st);
@@ -253,7 +261,7 @@ __device__ __forceinline__ void lines_tile(const LinesArgs &a, int bx, long long
             if (act) {
                 for (int p = sub; p < n; p += a.tpl) {
                     const cfx q = fx_mul_s(buf[p * ld + l], Sl[(long long)(p <= a.half ? p : h2 - p) * a.s_pos], ke,
-                                           neg_b ^ (p > a.half ? neg_z : 0), near);
+                                           neg_b ^ (p > a.half ? neg_z : 0), eS > -900);
                     buf[p * ld + l] = odd == 0 ? q : cfx{q.y, -q.x};
                 }
                 if (sub == 0) tl.eo[l] = 2 * tile_div(a.st) - sc.ke - ke, tl.bad[l] = bad;
@@ -482,7 +490,7 @@ __device__ __forceinline__ void c2r_tile(const RowsArgs &a, int bx, unsigned cha
     if constexpr (FX) {
         // the inputs' bounds hold for Z / 4 (|Z| / 4 <= the mean of |X[k]| and |X[N-k]|)
         const FxScale sc = tile_scale(buf, ld, np, a.st, 62, l, sub, a.tpl, act, tl);
-        if (act && sub == 0) tl.eo[l] = tile_div(a.st) + 2 - sc.ke, tl.bad[l] = sc.bad;
+        if (act && sub == 0) tl.eo[l] = tile_div(a.st) + 2 - sc.ke + a.exp, tl.bad[l] = sc.bad;
         __syncthreads();
     }
     if (act) {
