@@ -481,7 +481,7 @@ FSP_CFGX(512, 8, 4, 8, 8, 8)
 FSP_CFGX(1024, 16, 4, 16, 8, 8)
 #undef FSP_CFGX
 // Rows: lengths 64 and 256 run faster in two stages (P1 / P5 at N = 256 0.161 /
-// 0.152 ms with 16*16, 0.166 / 0.162 with 8*4*8)
+// 0.154 ms with 16*16, 0.166 / 0.162 with 8*4*8)
 template <int N> struct RowX : CfgX<N> {};
 template <> struct RowX<64> {
     static constexpr int V = 8, L = 16, R1 = 8, R2 = 8, R3 = 1;
