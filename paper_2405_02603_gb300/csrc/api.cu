@@ -672,10 +672,12 @@ bool plan_live(const fsp_plan *p) {
     return p && g_plans.count(p) && p->magic == kMagic;
 }
 
-// The order of a spectrum as a power of two, 0 within 2^+-50.
+// The power of two to divide a spectrum of the order of x by: none within 2^+-50,
+// else what brings it to 2^+-40.  (Not to 1: kept on its side, the passes between
+// P2 and P5 stay within the range that the true spectrum gives them.)
 int order_of(double x) {
     const int e = x > 0.0 && std::isfinite(x) ? std::ilogb(x) : 0;
-    return std::abs(e) < 50 ? 0 : std::min(1000, std::max(-1000, e));
+    return std::abs(e) < 50 ? 0 : std::min(1000, std::max(-1000, e > 0 ? e - 40 : e + 40));
 }
 // s_exp and f_exp of an FP64 plan: h^3 / (8 n_x n_y n_z) times the box's integral of
 // 1 / 4 pi r (L^2 within a few octaves; Hockney-Eastwood also has its value at the

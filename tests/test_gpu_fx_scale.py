@@ -94,3 +94,14 @@ def test_spectrum_batch_and_slabs(fsp, N):
         batch.close()
     check(fsp.solve_noalloc(torch.from_numpy(S).cuda(), rho, phi), want)
     check(fsp.solve_distributed_local(N, rho, L, "vg_dct", "f64", 3), want)
+
+
+@pytest.mark.parametrize("N", [32, 30])
+def test_largest_sources(fsp, N):
+    """What overflows is what overflowed: a source close to the range's end in a
+    box whose spectrum is small."""
+    import torch
+    p = fsp.Plan(N, 2.0 ** -60, "vg_dct", "f64")
+    rho = torch.full((N, N, N), 1.0, dtype=torch.float64, device="cuda")
+    top = 2.0 ** (1023 - 2 * int(np.ceil(np.log2(N))))  # the second pass holds N^2 of it
+    check(p.solve(rho * top), p.solve(rho) * top)
